@@ -52,6 +52,7 @@ struct GraphView {
   const uint64_t* rrow_off;  // [n+1] in-edge CSR or nullptr
   const uint2* redges;       // [m] {source, cost}, rows sorted by (cost, source)
   const uint2* rowdeg;       // [n] {start of out-row, out-degree} (m < 2^32)
+  uint32_t max_w;            // largest edge cost (0 without edges)
 };
 
 // Per-vertex record gathered by the selection and relax steps: the tentative
@@ -112,9 +113,7 @@ struct Ctl {
   int err;                  // sssp_status recorded by a device-side failure
   unsigned int gate;        // solo mode: bumped when the leader hands back to the group
   unsigned long long heartbeat;  // solo mode: phases done by the leader (progress for waiters)
-  unsigned long long next_phase; // solo mode: phase the group resumes at
-  unsigned int resume_relax;     // solo mode: 1 = the group resumes at the relax step of next_phase
-  unsigned int pad;
+  unsigned long long next_phase; // solo mode: 2 k + 1 if the group resumes at the relax step of phase k, 2 k at its start
   GridBarrier bar;
   // near/far split: far fringe vertices, a work counter and two key
   // histograms (use u fills hist[u & 1] while the other one is cleared)

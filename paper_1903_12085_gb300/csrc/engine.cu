@@ -33,13 +33,15 @@
 //     by OUT-SIMPLE (out-minima grow when a target settles) and DIJK.
 //
 // Solo mode: while |F| is small, block 0 of the group runs whole phases alone
-// with block barriers (tens of ns instead of ~1 us per grid barrier); the other
-// blocks wait on a bounded gate and rejoin when |F| grows or the solve ends.
+// with the fringe in shared memory and block barriers (tens of ns instead of ~1
+// us per grid barrier); the other blocks wait on a bounded gate and rejoin when
+// |F| grows or the solve ends.
 //
 // Phase control: the phase that settles the source is phase 1; the loop ends
 // when the next queue is empty.
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -49,6 +51,19 @@
 #include "policy.cuh"
 
 namespace sssp {
+
+#define SSSP_RARE(x) __builtin_expect(!!(x), 0)
+
+// What a kernel instance serves.  kAny: everything.  kArms: fused thresholds on
+// any of a policy's arms (IN-STATIC or IN-SIMPLE, sparse or dense), costs up to
+// kSoloNarrowW, nothing to record (trace, settle phases).  kStatic: the same on
+// static minima and the sparse queue alone.  They are kernels of their own: a
+// taken branch to code that is not in the instruction buffer costs 75 to 100
+// cycles (25 if it is; measured) and a phase takes dozens of them, and the
+// registers a step may use without saving them first depend on every other
+// function of its kernel.  (R-MAT s22 on the static criteria: 9.3 ms in an
+// instance that serves everything, 8.9 in its own.)
+enum { kAny = 0, kArms = 1, kStatic = 2 };
 
 // A group of co-resident blocks running one solve.  size == 1: block barriers.
 struct Grp {
@@ -202,9 +217,16 @@ struct Shared {
   uint32_t* whist;            // kWarps * kNfRing: per-warp bucket-list counts of a relax tile
 };
 
-__device__ __forceinline__ Shared carve(unsigned char* smem) {
+// The dynamic shared memory of a block.  Every step names it (and the block's
+// state below) itself instead of taking a pointer to it: an address that
+// arrives as an argument of an out-of-line function is generic, and its loads
+// and stores then cost a global access's issue and scoreboard instead of a
+// shared-memory one's.
+extern __shared__ __align__(16) unsigned char smem_all[];
+
+__device__ __forceinline__ Shared carve() {
   Shared s;
-  s.red = reinterpret_cast<unsigned long long*>(smem);
+  s.red = reinterpret_cast<unsigned long long*>(smem_all);
   s.bases = s.red + 64;
   s.s_d = s.bases + 2;
   s.s_base = reinterpret_cast<uint32_t*>(s.s_d + kWarps * kTile);
@@ -283,19 +305,47 @@ __device__ __forceinline__ Arm arm_for(const SolveParams& p, uint32_t nF) {
 // policy network on the phase-start features, evaluated by warp 0 of the block
 // and shared through shared memory.  Every thread of the block calls it; every
 // block computes the same arm from the same inputs.
-static_assert(kPolWeights * sizeof(float) == kSmemBytes - kPolicySmemOffset, "policy smem size");
+static_assert(kPolWeights * sizeof(float) == kPolicySmem, "policy smem size");
 
 // The policy weights staged in dynamic shared memory by solve_body.
-__device__ __forceinline__ const float* policy_smem() {
-  extern __shared__ __align__(16) unsigned char smem_all[];
-  return reinterpret_cast<const float*>(smem_all + kPolicySmemOffset);
+__device__ __forceinline__ const float* policy_smem(const SolveParams& p) {
+  return reinterpret_cast<const float*>(smem_all + p.pol_off);
+}
+
+// Largest fringe an episode on one block starts with, and goes on with.  A
+// limit below kSoloCap is the caller's own; otherwise an episode may use every
+// slot, and starts with some free (each phase needs one per edge it relaxes).
+// With a policy both are the limit itself, so that the phases in which the
+// network is asked do not depend on how many slots a launch has.
+__device__ __forceinline__ uint32_t solo_limit(const SolveParams& p, uint32_t eighths) {
+  const bool policy = (p.crit & SSSP_POLICY_LEARNED) != 0;
+  return p.solo_max < kSoloCap || policy ? min(p.solo_max, kSoloCap) : p.solo_spt * blockDim.x / 8 * eighths;
+}
+__device__ __forceinline__ uint32_t solo_enter(const SolveParams& p) { return solo_limit(p, 5); }
+__device__ __forceinline__ uint32_t solo_stay(const SolveParams& p) { return solo_limit(p, 6); }
+
+static __shared__ SolveParams s_p;
+
+// The network's choice on the phase-start features, by one warp.  Out of line
+// and called by that warp alone: inlined it made the phase loops longer by its
+// whole length, and as a function of all threads it had them save what they hold.
+// Its time is its length with cold instruction caches: about 1.4 us where scalar
+// weight loads, a reduction of each output and a second division took 2.1.
+static __shared__ int s_arm;
+__device__ __noinline__ void policy_eval(uint32_t nF, uint64_t k, uint32_t e_prev, uint32_t s_prev, uint32_t f_prev) {
+  __shared__ __align__(16) float s_act[2 * kPolHidden];
+  const SolveParams& p = s_p;
+  float y[kPolArms];
+  const float f = policy_feature_lane(nF, p.g.n, (uint32_t)p.g.m, (uint32_t)k, e_prev, s_prev, f_prev);
+  policy_forward_warp(policy_smem(p), f, s_act, y);
+  if ((threadIdx.x & 31) == 0) s_arm = policy_pick(y, p.ws.cur_in != nullptr, (uint64_t)nF * 32 >= p.g.n);
 }
 
 // split = true (the fringe is split into near and far parts) fixes arm 0,
 // IN-STATIC on the sparse queue: the split exists for large fringes, where the
 // queue scan is what it saves, and IN-SIMPLE cannot use its static keys.
 // nQ: queue length (the dense/sparse choice without a policy); nF: |F|.
-__device__ Arm choose_arm(const SolveParams& p, uint64_t k, uint32_t nQ, uint32_t nF, uint64_t e_prev,
+__device__ __forceinline__ Arm choose_arm(const SolveParams& p, uint64_t k, uint32_t nQ, uint32_t nF, uint64_t e_prev,
                           uint64_t s_prev, uint64_t f_prev, bool split) {
   if (!(p.crit & SSSP_POLICY_LEARNED) || p.policy == nullptr) return arm_for(p, nQ);
   if (split) {
@@ -305,20 +355,13 @@ __device__ Arm choose_arm(const SolveParams& p, uint64_t k, uint32_t nQ, uint32_
     a.index = 0;
     return a;
   }
-  __shared__ int s_arm;
-  if ((threadIdx.x >> 5) == 0) {
-    float f[kPolFeat], y[kPolArms];
-    policy_features(f, nF, p.g.n, p.g.m, k, e_prev, s_prev, f_prev);
-    policy_forward_warp(policy_smem(), f, y);
-    if (threadIdx.x == 0) s_arm = policy_pick(y, p.ws.cur_in != nullptr, (uint64_t)nF * 32 >= p.g.n);
-  }
+  if ((threadIdx.x >> 5) == 0) policy_eval(nF, k, (uint32_t)e_prev, (uint32_t)s_prev, (uint32_t)f_prev);
   __syncthreads();
   Arm a;
   a.index = s_arm;
   a.in_simple = a.index >= 2;
   a.dense = (a.index & 1) != 0;
-  __syncthreads();
-  return a;
+  return a;  // (the next choice is at least a phase, with its barriers, away)
 }
 
 // Trace arm bits of the near/far split: split active in the phase; the far
@@ -354,6 +397,15 @@ struct NfView {
   unsigned int* cnt;          // [kNfRing] list fills
   unsigned int* beyond;       // lowest bucket with an unlisted far vertex
 };
+
+// A block's state while it works on a solve, the same for all its threads: the
+// solve's parameters (s_p, above), its group (s_grp1: this block alone), mode,
+// running counters (thread 0 of the leading block) and near/far view.
+static __shared__ Grp s_grp, s_grp1;
+static __shared__ Mode s_md;
+static __shared__ Stats s_st;
+static __shared__ NfView s_nv;
+static __shared__ uint32_t s_nf_uses;  // key histograms used so far
 
 // Bucket of a far vertex's stored word (key > B >= O).
 __device__ __forceinline__ uint32_t nf_bucket(const NfView& nv, unsigned long long word, uint32_t im) {
@@ -440,7 +492,7 @@ __device__ __forceinline__ void nf_list_append_n(const NfView& nv, const uint32_
 // queue by the one relaxation whose atomicMin saw the bit go.  `fresh` asks the
 // caller to append t to the next queue.  kNF = false is the same code for a
 // solve with no far vertex (B = kNoBound).
-template <bool kNF>
+template <bool kNF, int kKind>
 __device__ __forceinline__ void relax_edge_rec(const SolveParams& p, const Mode& md, uint32_t t, uint32_t cost,
                                                unsigned long long du, const VRec& rt, const NfView& nv,
                                                unsigned long long& pd, unsigned long long& po, bool& fresh,
@@ -455,7 +507,7 @@ __device__ __forceinline__ void relax_edge_rec(const SolveParams& p, const Mode&
     if (rt.d == kUnexplored) {
       old = atomicMin(&w.vrec[t].d, enc);
       if (old == kUnexplored) {
-        if (status_live(md, kNF)) w.status[t] = kF;
+        if (kKind != kStatic && status_live(md, kNF)) w.status[t] = kF;
         if (kNF && (enc & kFarBit)) {
           ++dfar;
           if (nv.lists) app = nf_bucket(nv, enc, rt.im);
@@ -482,7 +534,7 @@ __device__ __forceinline__ void relax_edge_rec(const SolveParams& p, const Mode&
         if (b != nf_bucket(nv, rt.d, rt.im)) app = b;
       }
     }
-    if (md.fused && enc < old) {
+    if ((kKind != kAny || md.fused) && enc < old) {
       pd = cand < pd ? cand : pd;
       if (rt.om != kInf32) {
         const unsigned long long x = cand + rt.om;
@@ -492,13 +544,16 @@ __device__ __forceinline__ void relax_edge_rec(const SolveParams& p, const Mode&
   }
 }
 
-// The same with t's record loaded here (rt above is the record as read
-// before any update of this relaxation).
-template <bool kNF>
-__device__ __forceinline__ void relax_edge(const SolveParams& p, const Mode& md, uint32_t t, uint32_t cost,
-                                           unsigned long long du, const NfView& nv, unsigned long long& pd,
-                                           unsigned long long& po, bool& fresh, int& dfar, uint32_t& app) {
-  relax_edge_rec<kNF>(p, md, t, cost, du, ldcg_vrec(&p.ws.vrec[t]), nv, pd, po, fresh, dfar, app);
+// threadIdx.x and blockDim.x, read anew wherever it is called (volatile).
+__device__ __forceinline__ unsigned int opaque_tid() {
+  unsigned int x;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(x));
+  return x;
+}
+__device__ __forceinline__ unsigned int opaque_nthr() {
+  unsigned int x;
+  asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(x));
+  return x;
 }
 
 // Relax-list entry `slot` covers edges [base, base + deg) of the phase's edge
@@ -517,6 +572,7 @@ __device__ __forceinline__ void mark_tile_owner(uint32_t* owner, uint32_t slot, 
 struct PhaseHead {
   uint32_t nQ;
   uint32_t far;
+  uint32_t e_prev;  // edges of the last phase
   unsigned long long min_d, min_out;
   bool split;  // near/far split active (from the block's own state)
 };
@@ -527,6 +583,7 @@ __device__ __forceinline__ PhaseHead load_head(const Ctl* ctl, uint64_t k, bool 
   h.split = split;
   h.nQ = ldcg_u32(&S0->qcount);
   h.far = ldcg_u32(&ctl->far_count);
+  h.e_prev = (uint32_t)ldcg_u64(&ctl->slot[(k + 3) % 4].relax_packed);
   h.min_d = min(ldcg_u64(&S0->min_d), ldcg_u64(&S0->a_min_d));
   h.min_out = min(ldcg_u64(&S0->min_out), ldcg_u64(&S0->a_min_out));
   return h;
@@ -535,13 +592,18 @@ __device__ __forceinline__ PhaseHead load_head(const Ctl* ctl, uint64_t k, bool 
 // ---------------------------------------------------------------------------
 // Step B of phase k (after step A for the three-step kind), by every block of
 // the group, ending with a group barrier.  Returns false if a barrier gave up.
-__device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, const Mode& md, const Arm arm, uint64_t k,
-                                          const PhaseHead& h, const Shared& sh, Stats& st) {
+template <int kKind>
+__device__ __noinline__ bool phase_select(bool alone, const Arm arm, uint64_t k, const PhaseHead h) {
+  const SolveParams& p = s_p;
+  const Grp& grp = alone ? s_grp1 : s_grp;
+  const Mode& md = s_md;
+  Stats& st = s_st;
+  const Shared sh = carve();
   const GraphView& g = p.g;
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
   const uint32_t n = g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr();
   const unsigned int lane = tid & 31;
   const uint64_t gthreads = (uint64_t)grp.size * nthr;
   const uint64_t gtid = (uint64_t)grp.rank * nthr + tid;
@@ -552,20 +614,21 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
   PhaseSlot* S0 = &ctl->slot[k % 4];
   PhaseSlot* S1 = &ctl->slot[(k + 1) % 4];
   const uint32_t nF = h.nQ;
-  const bool wstat = status_live(md, h.split);
-  const bool dense = arm.dense;
-  const bool in_dyn = md.use_in && arm.in_simple && w.cur_in != nullptr;
+  const bool wstat = kKind != kStatic && status_live(md, h.split);
+  const bool dense = kKind != kStatic && arm.dense;
+  const bool fused = kKind != kAny || md.fused, settle = kKind == kAny && w.settle_phase != nullptr;
+  const bool in_dyn = kKind != kStatic && md.use_in && arm.in_simple && w.cur_in != nullptr;
   if (leader) {
     reset_slot(&ctl->slot[(k + 2) % 4]);
     const uint32_t fs = nF + (md.nearfar ? h.far : 0u);
     S0->fsize = fs;
     st.sum_f += fs;
-    if (w.trace) S0->t_start = globaltimer_ns();
+    if (kKind == kAny && w.trace) S0->t_start = globaltimer_ns();
   }
 
   // ---- thresholds
   unsigned long long minD, minOut, min_apx = kInf64;
-  if (md.fused) {
+  if (fused) {
     minD = h.min_d;
     minOut = h.min_out;
     if (in_dyn) {
@@ -659,7 +722,7 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
     if (md.approx) min_apx = ldcg_u64(&S0->a_min_apx);
   }
   uint32_t amin = kInf32;
-  if (md.dijk) {  // DIJK: the lowest id among fringe vertices of minimum d
+  if (kKind == kAny && md.dijk) {  // DIJK: the lowest id among fringe vertices of minimum d
     uint32_t lid = kInf32;
     if (dense) {
       for (uint64_t v = gtid; v < n; v += gthreads)
@@ -724,7 +787,7 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
       const unsigned long long dv = rr[j].d;
       bool sel = false;
       if (md.use_in) {
-        if (md.in_full) {
+        if (kKind == kAny && md.in_full) {
           const unsigned long long im = ldcg_u64(&w.im_full[v]);
           sel = (im == kInf64) || dv <= minD + im;
         } else {
@@ -733,20 +796,20 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
         }
       }
       if (!sel && md.use_out) sel = dv <= minOut;
-      if (!sel && md.approx) {
+      if (kKind == kAny && !sel && md.approx) {
         const unsigned long long ai = ldcg_u64(&w.apx_in[v]);
         sel = ai == kInf64 || dv <= minD + ai || dv <= min_apx;
       }
-      if (!sel && md.dijk) sel = (v == amin);
+      if (kKind == kAny && !sel && md.dijk) sel = (v == amin);
       if (sel) {
         if (wstat) w.status[v] = kS;
         w.vrec[v].d = dv | kSettledBit;
-        if (w.settle_phase) w.settle_phase[v] = (uint32_t)k;
+        if (settle) w.settle_phase[v] = (uint32_t)k;
         rd[j] = __ldg(&g.rowdeg[v]);
         selm |= 1u << j;
       } else {
         keepm |= 1u << j;
-        if (md.fused) {
+        if (fused) {
           pd = dv < pd ? dv : pd;
           if (rr[j].om != kInf32) {
             const unsigned long long x = dv + rr[j].om;
@@ -785,17 +848,17 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
     for (int j = 0; j < kSelItems; ++j) {
       if ((keepm >> j) & 1u) {
         const uint32_t slot = kbase + __popc(kb[j] & lt);
-        if (slot < n) Qn[slot] = vv[j];
+        if (!SSSP_RARE(slot >= n)) Qn[slot] = vv[j];
         else atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
       }
       kbase += __popc(kb[j]);
       if ((rb[j] >> lane) & 1u) {
         const uint32_t slot = rslot + __popc(rb[j] & lt);
         const uint32_t eb = ebase + eincl[j] - rd[j].y;
-        if (slot < n) {
+        if (!SSSP_RARE(slot >= n)) {
           *reinterpret_cast<ulonglong2*>(&w.sp[slot]) =
               make_ulonglong2(rr[j].d, (unsigned long long)rd[j].x | ((unsigned long long)eb << 32));
-          if (w.tile_owner) {
+          if (kKind != kAny || w.tile_owner) {
             const uint64_t t0 = ((uint64_t)eb + kTile - 1) / kTile;  // first tile starting inside [eb, eb + deg)
             if (t0 * kTile < (uint64_t)eb + rd[j].y) {
               w.tile_owner[t0] = slot;
@@ -809,7 +872,7 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
       rslot += __popc(rb[j]);
       ebase += __shfl_sync(0xFFFFFFFFu, eincl[j], 31);
     }
-    if (w.tile_owner && __any_sync(0xFFFFFFFFu, wide != 0)) {
+    if ((kKind != kAny || w.tile_owner) && __any_sync(0xFFFFFFFFu, wide != 0)) {
       // recompute each wide entry's slot and edge range and share it
       uint32_t rs = (uint32_t)(rbase >> 32), es = (uint32_t)rbase;
 #pragma unroll
@@ -831,7 +894,7 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
   }
   settled_here = __reduce_add_sync(0xFFFFFFFFu, settled_here);
   if (lane == 0 && settled_here) atomicAdd(&S0->settled_now, settled_here);
-  if (md.fused) block_min2_to_global(pd, po, &S1->min_d, md.use_out ? &S1->min_out : nullptr, sh.red);
+  if (fused) block_min2_to_global(pd, po, &S1->min_d, md.use_out ? &S1->min_out : nullptr, sh.red);
   return grp.sync();
 }
 
@@ -846,14 +909,19 @@ __device__ __noinline__ bool phase_select(const SolveParams& p, const Grp& grp, 
 // each of its kRelaxItems edges by binary search there, issues all of its edge
 // loads, then all of its target-record loads, and relaxes.  Vertices new to
 // the next queue get their slots from one atomicAdd per tile.
-template <bool kNF>
-__device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, const Mode& md, const Arm arm, uint64_t k,
-                                         const NfView& nv, bool resumed, const Shared& sh, Stats& st) {
+template <bool kNF, int kKind>
+__device__ __noinline__ bool phase_relax(bool alone, const Arm arm, uint64_t k, bool resumed) {
+  const SolveParams& p = s_p;
+  const Grp& grp = alone ? s_grp1 : s_grp;
+  const Mode& md = s_md;
+  const NfView& nv = s_nv;
+  Stats& st = s_st;
+  const Shared sh = carve();
   const GraphView& g = p.g;
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
   const uint32_t n = g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr();
   const unsigned int lane = tid & 31, warp = tid >> 5;
   const bool leader = grp.rank == 0 && tid == 0;
   const int cur = (int)((k - 1) & 1);
@@ -871,14 +939,17 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
   const uint64_t tile0 = (uint64_t)grp.rank * nwarps + warp;
   const uint64_t owner_len = g.m / kTile + 2;  // length of the tile-owner array
   uint32_t mlo = 0, mhi = 0;  // owner marks of the next tile to stage
-  if (w.tile_owner && tile0 + 1 < owner_len) {
+  const bool marks = kKind != kAny || w.tile_owner != nullptr, approx = kKind == kAny && md.approx;
+  const bool trace = kKind == kAny && w.trace != nullptr;
+  const bool fused = kKind != kAny || md.fused;
+  if (marks && tile0 + 1 < owner_len) {
     mlo = ldcg_u32(&w.tile_owner[tile0]);
     mhi = ldcg_u32(&w.tile_owner[tile0 + 1]);
   }
   const unsigned long long packed = ldcg_u64(&S0->relax_packed);
   const uint32_t nS = (uint32_t)(packed >> 32);
   const uint32_t E = (uint32_t)packed;
-  if (leader && w.trace && !resumed) S0->t_select = globaltimer_ns();  // (a hand-off set it)
+  if (trace && leader && !resumed) S0->t_select = globaltimer_ns();  // (a hand-off set it)
   const unsigned int lt = (1u << lane) - 1u;
   uint32_t* s_base = sh.s_base + warp * kTile;
   uint32_t* s_row = sh.s_row + warp * kTile;
@@ -897,7 +968,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
     const uint32_t e0 = (uint32_t)(t * kTile);
     const uint32_t e1 = (uint64_t)e0 + kTile < E ? e0 + kTile : E;
     uint32_t lo = 0, hi = nS - 1;
-    if (w.tile_owner) {
+    if (marks) {
       // entries lo .. hi intersect the tile (hi may start just past it, and is
       // then dropped by the kTile cap below: the per-edge search never picks it)
       lo = mlo;
@@ -937,7 +1008,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
   for (uint64_t tile = tile0; tile * kTile < E;) {
     const uint64_t next = tile + gwarps;
     const bool has_next = next * kTile < E;
-    if (has_next && w.tile_owner && next + 1 < owner_len) {
+    if (has_next && marks && next + 1 < owner_len) {
       mlo = ldcg_u32(&w.tile_owner[next]);
       mhi = ldcg_u32(&w.tile_owner[next + 1]);
     }
@@ -954,7 +1025,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
       tv[it] = ed[it].x;
       if ((valid >> it) & 1u) {
         bool fresh = false;
-        relax_edge_rec<kNF>(p, md, ed[it].x, ed[it].y, s_d[(ownp >> (8 * it)) & 0xFFu], rt[it], nv, pd, po, fresh,
+        relax_edge_rec<kNF, kKind>(p, md, ed[it].x, ed[it].y, s_d[(ownp >> (8 * it)) & 0xFFu], rt[it], nv, pd, po, fresh,
                             dfar, app[it]);
         if (fresh) fmask |= 1u << it;
       }
@@ -967,7 +1038,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
     unsigned int fslot = 0, xslot = 0;
     if (nfr && lane == 0) {
       fslot = atomicAdd(&S1->qcount, nfr);
-      if (md.approx) xslot = atomicAdd(&S1->fresh_count, nfr);
+      if (approx) xslot = atomicAdd(&S1->fresh_count, nfr);
     }
     // ... and bucket-list ranges: ranks within the warp per ring slot
     // (shared-memory atomics), then one global atomicAdd per slot used, its
@@ -1012,9 +1083,9 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
         const unsigned int fb = __ballot_sync(0xFFFFFFFFu, (fmask >> it) & 1u);
         if ((fmask >> it) & 1u) {
           const uint32_t off = __popc(fb & lt);
-          if (fslot + off < n) Qn[fslot + off] = tv[it];
+          if (!SSSP_RARE(fslot + off >= n)) Qn[fslot + off] = tv[it];
           else atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
-          if (md.approx) {
+          if (approx) {
             if (xslot + off < n) w.fresh[xslot + off] = tv[it];
             else atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
           }
@@ -1040,7 +1111,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
     }
     tile = next;
   }
-  if (md.fused) block_min2_to_global(pd, po, &S1->min_d, md.use_out ? &S1->min_out : nullptr, sh.red);
+  if (fused) block_min2_to_global(pd, po, &S1->min_d, md.use_out ? &S1->min_out : nullptr, sh.red);
   if (kNF) {  // far-part count: one atomic per block (the barrier above orders scratch reuse)
     uint32_t tf;
     block_exclusive_scan((uint32_t)dfar, sh.scan, &tf);
@@ -1052,7 +1123,7 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
     st.settled += settled_now;
     st.relaxed += E;
     st.phases = k;
-    if (w.trace && k <= w.trace_cap) {
+    if (trace && k <= w.trace_cap) {
       const uint32_t code = ldcg_u32(&S0->arm);
       const bool in_dyn = md.use_in && w.cur_in != nullptr &&
                           ((code & 0x80u) ? ((code >> 8) >= 2) : arm.in_simple);
@@ -1083,415 +1154,675 @@ __device__ __noinline__ bool phase_relax(const SolveParams& p, const Grp& grp, c
 static __shared__ Arm s_arm_last;
 static __shared__ unsigned long long s_arm_k;
 
-__device__ __forceinline__ bool run_phase(const SolveParams& p, const Grp& grp, const Mode& md, uint64_t k,
-                                          const NfView& nv, uint32_t nf_code, const PhaseHead& h, const Shared& sh,
-                                          Stats& st) {
-  Arm arm;
-  if ((p.crit & SSSP_POLICY_LEARNED) && p.policy != nullptr) {
-    // The network is evaluated in the first grid phase of a solve and then at
-    // most every 4th phase (its forward pass sits on the phase's critical
-    // path); the phases in between keep its last choice.  (The previous
-    // phase's counts are its features.)  Every block evaluates the same inputs.
-    if (nv.bound != kNoBound) {
-      arm = choose_arm(p, k, h.nQ, 0, 0, 0, 0, true);  // split: the static sparse arm
-    } else if (k <= s_arm_k || k - s_arm_k >= 4) {
-      const PhaseSlot* prev = &p.ws.ctl->slot[(k + 3) % 4];
-      arm = choose_arm(p, k, h.nQ, h.nQ + (md.nearfar ? h.far : 0u), (uint32_t)ldcg_u64(&prev->relax_packed),
-                       ldcg_u32(&prev->settled_now), ldcg_u32(&prev->fsize), false);
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        s_arm_last = arm;
-        s_arm_k = k;
-      }
-      __syncthreads();
-    } else {
-      arm = s_arm_last;
-    }
-  } else {
-    arm = arm_for(p, h.nQ);
-  }
-  if (grp.rank == 0 && threadIdx.x == 0) p.ws.ctl->slot[k % 4].arm = arm_code(arm, grp.size == 1) | nf_code;
-  if (!phase_select(p, grp, md, arm, k, h, sh, st)) return false;
-  return nv.bound != kNoBound ? phase_relax<true>(p, grp, md, arm, k, nv, false, sh, st)
-                              : phase_relax<false>(p, grp, md, arm, k, nv, false, sh, st);
-}
-
-// Relax step of a solo phase: the warps of the block stride over the relax
-// list's edges; vertices new to the next queue get slots from a shared counter
-// (slots past kSoloCap go to the global queue at the same index).
-struct SoloRelax {
-  const unsigned long long* sp_d;
-  const uint32_t* sp_row;
-  const uint32_t* sp_base;
-  uint32_t nS, E;
-  uint32_t* sqn;
-  uint32_t* gqn;
-  unsigned int* qn;
-};
-
-template <bool kNF>
-__device__ __forceinline__ void solo_relax(const SolveParams& p, const Mode& md, const SoloRelax& r,
-                                           const NfView& nv, unsigned long long& pd, unsigned long long& po,
-                                           int& dfar) {
-  const unsigned int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t eb = warp * 32; eb < r.E; eb += blockDim.x) {
-    const uint32_t e = eb + lane;
-    bool fresh = false;
-    uint32_t t = 0, app = kNoBucket;
-    if (e < r.E) {
-      uint32_t a = 0, b = r.nS;
-      while (b - a > 1) {
-        const uint32_t mid = (a + b) >> 1;
-        if (r.sp_base[mid] <= e) a = mid; else b = mid;
-      }
-      const uint2 ed = __ldg(&p.g.edges[r.sp_row[a] + (e - r.sp_base[a])]);
-      t = ed.x;
-      relax_edge<kNF>(p, md, t, ed.y, r.sp_d[a], nv, pd, po, fresh, dfar, app);
-    }
-    if (kNF) nf_list_append(nv, app, t);
-    const unsigned int fmask = __ballot_sync(0xFFFFFFFFu, fresh);
-    if (fmask) {
-      unsigned int b0 = 0;
-      if (lane == 0) b0 = atomicAdd(r.qn, (unsigned int)__popc(fmask));
-      b0 = __shfl_sync(0xFFFFFFFFu, b0, 0);
-      if (fresh) {
-        const uint32_t slot = b0 + __popc(fmask & ((1u << lane) - 1u));
-        if (slot < kSoloCap) r.sqn[slot] = t;
-        else if (slot < p.g.n) r.gqn[slot] = t;
-        else atomicCAS(&p.ws.ctl->err, 0, (int)SSSP_ERR_INTERNAL);
-      }
-    }
-  }
-}
-
-// Solo episode (fused thresholds only): this block runs phases k, k+1, ...
-// alone while |F| <= min(solo_max, kSoloCap).  The two fringe queues, the
-// relax list, the counters and the thresholds live in shared memory; global
-// memory is touched only for vertex records, status bytes, edges and distance
-// updates.  Queue slots at or beyond kSoloCap go to the global queue at the
-// same index.  If a phase's relax list has more than solo_edges edges and
-// `can_handoff`, the episode stops after the selection and hands the relax step
-// to the whole group (*handoff = true).
-// Entry: global queue q[(k-1)&1] with slot[k%3].qcount entries, thresholds in
-// slot[k%3].  Exit at phase k: the same state with slot[(k+1)%3] reset (no
-// handoff), or the state after a grid selection step of phase k (handoff).
-// All threads of the block call it.
-__device__ __forceinline__ uint64_t solo_episode(const SolveParams& p, const Mode& md_shared, uint64_t k, const NfView& nv,
-                                 uint32_t nf_code, unsigned char* smem, Stats& st_shared, bool can_handoff,
-                                 bool* handoff) {
-  const Mode md = md_shared;  // in registers for the episode (read in every step)
-  const GraphView& g = p.g;
-  const SolveWS& w = p.ws;
-  Ctl* ctl = w.ctl;
-  const uint32_t n = g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
-  const unsigned int lane = tid & 31, warp = tid >> 5;
-  unsigned long long* red = reinterpret_cast<unsigned long long*>(smem);
-  uint32_t* sqa = reinterpret_cast<uint32_t*>(red + 64);
-  uint32_t* sqb = sqa + kSoloCap;
-  unsigned long long* sp_d = reinterpret_cast<unsigned long long*>(sqb + kSoloCap);
-  uint32_t* sp_row = reinterpret_cast<uint32_t*>(sp_d + kSoloCap);
-  uint32_t* sp_base = sp_row + kSoloCap;
-  // (thread t loads the records of fringe entries t, t + blockDim, ... into
-  // registers and decides those same entries: no block barrier between)
-  static_assert(kSoloCap % kThreads == 0, "solo entries per thread");
-  // per-phase counters, double-buffered by phase parity: the buffer of phase
-  // k + 1 is cleared during phase k, after every thread has read it as phase
-  // k - 1's
-  __shared__ unsigned int s_qn[2], s_settled[2];
-  __shared__ unsigned int s_wk[32], s_wr[32], s_we[32];  // per-warp counts
-  __shared__ unsigned long long s_relax[2], s_thr_d[2], s_thr_o[2];
-  __shared__ int s_dfar[2];
-  *handoff = false;
-
-  const uint32_t cap = p.solo_max < kSoloCap ? p.solo_max : kSoloCap;
-  // counters of the previous phase (policy features)
-  uint32_t e_prev = (uint32_t)ldcg_u64(&ctl->slot[(k + 3) % 4].relax_packed);
-  uint32_t s_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].settled_now);
-  uint32_t f_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].fsize);
-  uint32_t nF = ldcg_u32(&ctl->slot[k % 4].qcount);
-  const bool kNF = nv.bound != kNoBound;
-  uint32_t far = kNF ? ldcg_u32(&ctl->far_count) : 0u;  // far part of F (not in the queues)
-  Stats& st = st_shared;  // thread 0's running counters
-  __shared__ unsigned long long s_t0, s_tsel;  // thread 0's trace stamps
-  Arm arm{false, false, -1};
-  unsigned int since_pick = 0;
-  unsigned long long minD = min(ldcg_u64(&ctl->slot[k % 4].min_d), ldcg_u64(&ctl->slot[k % 4].a_min_d));
-  unsigned long long minOut = min(ldcg_u64(&ctl->slot[k % 4].min_out), ldcg_u64(&ctl->slot[k % 4].a_min_out));
-  {
-    const uint32_t* gq = w.q[(k - 1) & 1];
-    uint32_t* sq = ((k - 1) & 1) ? sqb : sqa;
-    for (uint32_t i = tid; i < nF; i += nthr) sq[i] = ldcg_u32(gq + i);
-  }
-  if (tid < 2) {
-    s_qn[tid] = 0;
-    s_settled[tid] = 0;
-    s_relax[tid] = 0;
-    s_thr_d[tid] = s_thr_o[tid] = kInf64;
-    s_dfar[tid] = 0;
+__device__ __noinline__ Arm policy_arm(uint64_t k, uint32_t nQ, uint32_t far) {
+  // The network is evaluated in the first grid phase of a solve and then at
+  // most every 4th phase (its forward pass sits on the phase's critical
+  // path); the phases in between keep its last choice.  (The previous
+  // phase's counts are its features.)  Every block evaluates the same inputs.
+  if (s_nv.bound != kNoBound) return choose_arm(s_p, k, nQ, 0, 0, 0, 0, true);  // split: the static sparse arm
+  if (k > s_arm_k && k - s_arm_k < 4) return s_arm_last;
+  const PhaseSlot* prev = &s_p.ws.ctl->slot[(k + 3) % 4];
+  const Arm arm = choose_arm(s_p, k, nQ, nQ + (s_md.nearfar ? far : 0u), (uint32_t)ldcg_u64(&prev->relax_packed),
+                             ldcg_u32(&prev->settled_now), ldcg_u32(&prev->fsize), false);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_arm_last = arm;
+    s_arm_k = k;
   }
   __syncthreads();
+  return arm;
+}
+
+template <int kKind>
+__device__ __forceinline__ bool run_phase(bool alone, uint64_t k, uint32_t nf_code, const PhaseHead& h) {
+  const bool policy = kKind != kStatic && (s_p.crit & SSSP_POLICY_LEARNED) && s_p.policy != nullptr;
+  const Arm arm = kKind == kStatic ? Arm{false, false, -1} : policy ? policy_arm(k, h.nQ, h.far) : arm_for(s_p, h.nQ);
+  if (kKind == kAny) {
+    const uint32_t size = alone ? 1u : s_grp.size, rank = alone ? 0u : s_grp.rank;
+    if (rank == 0 && threadIdx.x == 0) s_p.ws.ctl->slot[k % 4].arm = arm_code(arm, size == 1) | nf_code;
+  }
+  if (!phase_select<kKind>(alone, arm, k, h)) return false;
+  return s_nv.bound != kNoBound ? phase_relax<true, kKind>(alone, arm, k, false)
+                                : phase_relax<false, kKind>(alone, arm, k, false);
+}
+
+// Solo episode (fused thresholds only): one block runs phases k, k+1, ...
+// alone while the fringe fits the slots it keeps in shared memory.  A fringe
+// vertex lives in a slot {D, minima, v, out-row}; its record in device memory
+// holds the slot's number instead of d, so a relaxation that finds a small
+// number there lowers the slot's D (a shared-memory atomic), one that finds an
+// unexplored vertex claims it for a free slot with one compare-and-swap, and
+// the selection and the thresholds never leave the SM.  (No other word looks
+// like a slot number: settled vertices have bit 63 set, far and unexplored
+// ones bit 62, and every near fringe vertex has a slot during the episode.)
+//
+// A phase is bound by its longest chain of instructions and round trips, not by
+// throughput, so both are kept few.  D is d less a base that follows minD: 32
+// bits hold it while no edge costs more than kSoloNarrowW (T = uint32_t; the
+// 64-bit version serves larger costs), which makes a slot one 16-byte load and
+// its tests a handful of instructions without a branch.  A thread tests the
+// slots tid, tid + blockDim, ... and a bit mask says which are in use, so
+// nothing is compacted.  Each warp deals the edges of the vertices it settled to
+// its lanes, the first 32 before the barrier between selection and relaxation,
+// which hides the edge loads behind it; there is no list of the whole block and
+// no atomic with a result.  New vertices go to the
+// free slots of another warp, a different one each phase, which keeps the warps'
+// shares of the fringe alike.  Two block barriers per phase; round trips to L2:
+// the edge, then the compare-and-swap with the target's minima and row beside
+// it.  On the 1024 x 1024 grid (34 thousand phases of 1,100 fringe vertices, 31
+// settled, 124 edges) a phase takes 3.3 us; with the fringe as a queue of
+// vertices, whose records, settled rows, edges, targets and claims were five
+// round trips and whose scan was bound by one SM's gathers, it took 6.0 us
+// (206 -> 114 ms a solve; 256 sources on the 512 x 512 grid 117 -> 72 ms).
+//
+// Entry: global queue q[(k-1)&1] with slot[k%4].qcount entries, thresholds in
+// slot[k%4].  Exit at phase k: the same state with slot[(k+1)%4] reset, or
+// (hand-off) the state after a grid selection step of phase k, when it relaxes
+// more edges than solo_edges allows, a warp has fewer free slots to fill than
+// edges to relax or settles more than kSoloList vertices, or a D nears the end
+// of its range.  All threads of the block call it.
+template <class T>
+struct SoloMem {
+  uint4* slot;   // {D (T = uint32_t), static in-minimum, static out-minimum, v}
+  uint2* row;    // {out-row start, out-degree}
+  T* wide;       // D (T = unsigned long long)
+  uint4* list;   // this warp's settled vertices: {out-row start, out-degree, D}
+  uint32_t* used;  // per thread: its slots in use
+  __device__ __forceinline__ T* d(uint32_t s) const {
+    return sizeof(T) == 4 ? reinterpret_cast<T*>(&slot[s].x) : &wide[s];
+  }
+};
+
+template <class T>
+__device__ __forceinline__ SoloMem<T> solo_carve() {
+  const uint32_t slots = s_p.solo_spt * blockDim.x;
+  SoloMem<T> m;
+  m.slot = reinterpret_cast<uint4*>(smem_all);
+  m.row = reinterpret_cast<uint2*>(m.slot + slots);
+  m.wide = reinterpret_cast<T*>(m.row + slots);
+  uint4* list = reinterpret_cast<uint4*>(m.wide + (sizeof(T) == 8 ? slots : 0));
+  m.list = list + (threadIdx.x >> 5) * kSoloList;
+  m.used = reinterpret_cast<uint32_t*>(list + (blockDim.x >> 5) * kSoloList);
+  return m;
+}
+
+// Counters of a solo phase, one set per phase parity: the set of phase k + 1
+// is cleared between the barriers of phase k, when no thread reads it any more.
+struct __align__(16) SoloCount {
+  uint32_t edges, settled, fresh, stop;  // stop: the phase is handed off
+  unsigned long long min_d, min_out;  // next phase's thresholds less the base (T-sized)
+  int far;
+  uint32_t heavy;  // the phase's edges are dealt out over the whole block
+  uint32_t room, pad;  // fewest free slots of a warp
+};
+static_assert(offsetof(SoloCount, min_d) == 16 && offsetof(SoloCount, room) == 40, "solo_clear, word by word");
+static __shared__ SoloCount s_sc[2];
+static __shared__ unsigned long long s_solo_n;  // hand-off and exit: entries written (and edges below them)
+
+// Where the policy's choice stands when an episode is interrupted only because
+// its slots or its edge list ran out (or by a hand-off within a single block):
+// the next episode goes on with it as if it had not been.
+static __shared__ Arm s_solo_arm;
+static __shared__ unsigned int s_solo_since, s_solo_cont;
+
+__device__ __forceinline__ uint32_t solo_warp_min(uint32_t x) { return __reduce_min_sync(0xFFFFFFFFu, x); }
+__device__ __forceinline__ unsigned long long solo_warp_min(unsigned long long x) { return warp_min_u64(x); }
+
+template <class T>
+__device__ __forceinline__ T* solo_thr(unsigned long long* x) { return reinterpret_cast<T*>(x); }
+
+__device__ __forceinline__ void solo_clear(SoloCount* c) {
+  c->edges = c->settled = c->fresh = c->stop = c->heavy = 0;
+  c->min_d = c->min_out = kInf64;
+  c->far = 0;
+  c->room = kInf32;
+}
+
+// Writes d back into the records of this thread's live slots and their vertices
+// to queue q (s_solo_n zeroed before, by a barrier).  All threads call it.
+template <class T>
+__device__ __forceinline__ void solo_write_back(const SoloMem<T>& m, uint32_t live, unsigned long long base,
+                                                uint32_t* q) {
+  const unsigned int lane = threadIdx.x & 31;
+  for (uint32_t j = 0; j < s_p.solo_spt; ++j) {
+    const bool on = (live >> j) & 1u;
+    const unsigned int bm = __ballot_sync(0xFFFFFFFFu, on);
+    if (!bm) continue;
+    uint32_t at = 0;
+    if (lane == 0) at = (uint32_t)atomicAdd(&s_solo_n, (unsigned long long)__popc(bm));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bm & ((1u << lane) - 1u));
+    if (on) {
+      const uint32_t s = j * blockDim.x + threadIdx.x, v = m.slot[s].w;
+      s_p.ws.vrec[v].d = base + *m.d(s);
+      q[at] = v;
+    }
+  }
+}
+
+// The state of a grid selection step of phase k, in global memory.  `sel`: the
+// slots this thread settled in it.  Leaves (entries << 32) | edges of the relax list
+// in s_solo_n.
+template <class T>
+__device__ __noinline__ void solo_hand_off(uint32_t k, uint32_t live, uint32_t sel, T od, T oo,
+                                           unsigned long long base, T minD, T minOut, uint32_t nF, uint32_t far,
+                                           uint32_t nf_code, unsigned long long t_start) {
+  const SolveWS& w = s_p.ws;
+  Ctl* const ctl = w.ctl;
+  SoloCount* const sc = &s_sc[k & 1];
+  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
+  const SoloMem<T> m = solo_carve<T>();
+  od = solo_warp_min(od);
+  oo = solo_warp_min(oo);
+  if ((tid & 31) == 0) {
+    atomicMin(solo_thr<T>(&sc->min_d), od);
+    atomicMin(solo_thr<T>(&sc->min_out), oo);
+  }
+  if (tid == 0) s_solo_n = 0;
+  __syncthreads();
+  solo_write_back(m, live, base, w.q[k & 1]);
+  __syncthreads();
+  if (tid == 0) s_solo_n = 0;
+  __syncthreads();
+  const unsigned int lane = tid & 31;
+  for (uint32_t j = 0; j < s_p.solo_spt; ++j) {
+    const uint32_t s = j * nthr + tid;
+    const uint2 row = (sel >> j) & 1u ? m.row[s] : make_uint2(0, 0);
+    const unsigned int bm = __ballot_sync(0xFFFFFFFFu, row.y > 0);
+    if (!bm) continue;
+    const uint32_t incl = warp_inclusive_scan(row.y);
+    unsigned long long at = 0;  // one packed add: the edge prefix is monotone in the entry
+    if (lane == 31) at = atomicAdd(&s_solo_n, ((unsigned long long)__popc(bm) << 32) | incl);
+    at = __shfl_sync(0xFFFFFFFFu, at, 31);
+    if (row.y > 0) {
+      const uint32_t i = (uint32_t)(at >> 32) + __popc(bm & ((1u << lane) - 1u)), eb = (uint32_t)at + incl - row.y;
+      *reinterpret_cast<ulonglong2*>(&w.sp[i]) =
+          make_ulonglong2(base + *m.d(s), (unsigned long long)row.x | ((unsigned long long)eb << 32));
+      if (w.tile_owner) mark_tile_owner(w.tile_owner, i, eb, row.y);
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    constexpr T inf = ~(T)0;
+    s_st.sum_f += nF + far;
+    ctl->far_count = far;
+    PhaseSlot* S0 = &ctl->slot[k % 4];
+    PhaseSlot* S1 = &ctl->slot[(k + 1) % 4];
+    reset_slot(S0);
+    reset_slot(S1);
+    reset_slot(&ctl->slot[(k + 2) % 4]);
+    S0->qcount = nF;
+    S0->fsize = nF + far;
+    S0->min_d = base + minD;
+    S0->min_out = minOut == inf ? kInf64 : base + minOut;
+    S0->relax_packed = s_solo_n;
+    S0->settled_now = sc->settled;
+    S0->arm = arm_code(s_solo_arm, true) | nf_code;
+    S0->t_start = t_start;
+    S0->t_select = globaltimer_ns();
+    S1->qcount = nF - sc->settled;
+    const T xd = *solo_thr<T>(&sc->min_d), xo = *solo_thr<T>(&sc->min_out);
+    if (xd != inf) S1->min_d = base + xd;
+    if (s_md.use_out && xo != inf) S1->min_out = base + xo;
+  }
+}
+
+// T = uint32_t: D is rebased once minD has moved this far from the base, and a
+// vertex settled with a D past the second limit (which static criteria never
+// reach: a fringe lies within twice the largest cost of its minD) ends the
+// episode, so that D + cost + minimum always fits.
+// A warp with more edges than kSoloHeavy makes the phase a heavy one: its edges
+// are dealt out over the whole block, at the price of two searches an edge.
+constexpr uint32_t kSoloHeavy = 64;
+constexpr uint32_t kSoloRebase = 1u << 30, kSoloLastD = 0xFFFFFFFEu - 2 * kSoloNarrowW;
+// Returns 4 k + kSoloResume (the relax step of phase k is handed to the group),
+// or + kSoloNoFit (the fringe's distances are too far apart: nothing was done).
+enum { kSoloResume = 1, kSoloNoFit = 2 };
+
+template <bool kNF, class T, int kKind>
+__device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool group) {
+  constexpr bool kNarrow = sizeof(T) == 4;
+  constexpr T inf = ~(T)0;
+  const SolveParams& p = s_p;
+  const SolveWS& w = p.ws;
+  const NfView& nv = s_nv;
+  VRec* const vrec = w.vrec;
+  const uint2* const edges = p.g.edges;
+  const uint2* const rowdeg = p.g.rowdeg;
+  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
+  const unsigned int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
+  const bool scribe = tid == nthr - 32;  // writes the trace
+  const uint32_t spt = p.solo_spt;       // slots per thread (at most 16)
+  const bool use_in = s_md.use_in, use_out = s_md.use_out;
+  uint8_t* const status = kKind != kStatic && status_live(s_md, kNF) ? w.status : nullptr;
+  const bool settle = kKind == kAny && w.settle_phase != nullptr, trace = kKind == kAny && w.trace != nullptr;
+  const bool policy = kKind != kStatic && (p.crit & SSSP_POLICY_LEARNED) != 0;
+  const SoloMem<T> m = solo_carve<T>();
+  __shared__ unsigned long long s_t0, s_tsel;  // trace stamps
+  __shared__ uint2 s_warp[32];  // per warp: edges of the phase, settled vertices
+  Ctl* const ctl = w.ctl;
+  uint32_t nF = ldcg_u32(&ctl->slot[k % 4].qcount);
+  uint32_t far = kNF ? ldcg_u32(&ctl->far_count) : 0u;  // far part of F (not in the slots)
+  unsigned long long base = 0;  // D = d - base
+  T minD, minOut;
+  {
+    const PhaseSlot* S0 = &ctl->slot[k % 4];
+    const unsigned long long d = min(ldcg_u64(&S0->min_d), ldcg_u64(&S0->a_min_d));
+    const unsigned long long o = min(ldcg_u64(&S0->min_out), ldcg_u64(&S0->a_min_out));
+    if (kNarrow) base = d;
+    minD = (T)(d - base);
+    minOut = o - base > inf ? inf : (T)(o - base);
+  }
+  unsigned int since_pick = s_solo_cont ? s_solo_since : 0u;
+  Arm arm = s_solo_cont ? s_solo_arm : Arm{false, false, -1};
+  // counters of the last phase (policy features), and of the episode
+  uint32_t e_prev = 0, s_prev = 0, f_prev = 0;
+  if (kKind != kStatic) {
+    e_prev = (uint32_t)ldcg_u64(&ctl->slot[(k + 3) % 4].relax_packed);
+    s_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].settled_now);
+    f_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].fsize);
+  }
+  unsigned long long sum_f = 0, sum_s = 0, sum_e = 0;
+  if (tid == 0) solo_clear(&s_sc[k & 1]);
+  uint32_t live = 0, spent = 0;  // this thread's fringe slots / those it settled in the last phase
+  {
+    const uint32_t* gq = w.q[(k - 1) & 1];
+    bool fits = true;
+    for (uint32_t j = 0; j < spt; ++j) {
+      const uint32_t s = j * nthr + tid;
+      if (s < nF) {
+        const uint32_t v = ldcg_u32(gq + s);
+        const VRec r = ldcg_vrec(&vrec[v]);
+        m.row[s] = __ldg(&rowdeg[v]);
+        m.slot[s] = make_uint4((uint32_t)(r.d - base), r.im, r.om, v);
+        if (!kNarrow) m.wide[s] = (T)r.d;
+        else if (r.d - base > kSoloLastD) fits = false;
+        live |= 1u << j;
+      } else {
+        *m.d(s) = inf;
+      }
+    }
+    m.used[tid] = live;
+    if (!__syncthreads_and(fits)) return 4ull * k + kSoloNoFit;
+    for (uint32_t b = live; b; b &= b - 1) {
+      const uint32_t s = (uint32_t)(__ffs(b) - 1) * nthr + tid;
+      vrec[m.slot[s].w].d = s;
+    }
+  }
+  if (tid == 0) s_solo_cont = 0;
+  T od, oo;
+  uint32_t sel;
+  bool hand = false, was_dyn = false;
+
   for (;;) {
-    const int pb = (int)(k & 1);  // this phase's counter buffer
-    const int cur = (int)((k - 1) & 1);
-    const uint32_t* sq = cur ? sqb : sqa;
-    uint32_t* sqn = cur ? sqa : sqb;
-    uint32_t* gqn = w.q[cur ^ 1];
+    SoloCount* const sc = &s_sc[k & 1];
     // the policy is evaluated on the first phase of the episode and every 8th
     // phase after it (the choice is logged per phase either way)
-    if (since_pick == 0) arm = choose_arm(p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
-    since_pick = (since_pick + 1) & 7u;
-    const bool in_dyn = md.use_in && arm.in_simple && w.cur_in != nullptr;
-    const uint32_t fs = nF + far;  // |F| at the start of the phase
-    if (tid == 0 && w.trace) s_t0 = globaltimer_ns();
-    // ---- B1: load the records of this thread's fringe entries (all in flight at once)
-    constexpr int kIt = kSoloCap / kThreads;
-    VRec r[kIt];
-#pragma unroll
-    for (int j = 0; j < kIt; ++j) {
-      const uint32_t i = tid + j * nthr;
-      if (i < nF) r[j] = ldcg_vrec(&w.vrec[sq[i]]);
+    if (kKind != kStatic && SSSP_RARE(since_pick == 0)) {
+      arm = choose_arm(p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
+      if (tid == 0) s_solo_arm = arm;
     }
-    if (in_dyn) {
-#pragma unroll
-      for (int j = 0; j < kIt; ++j) {
-        const uint32_t i = tid + j * nthr;
-        if (i < nF) r[j].im = in_min_dynamic(g, w, sq[i], false);
-      }
-    }
-    // IN-SIMPLE minima read status bytes that the selection below writes
-    if (in_dyn) __syncthreads();
-    // ---- B2: select.  Pass 1 decides and issues the row loads of the settled
-    // vertices; one block scan of per-warp counts gives every warp its output
-    // offsets; pass 2 writes the kept entries and the relax list (no shared
-    // atomics on the hot counters).
-    unsigned long long pd = kInf64, po = kInf64;
-    uint32_t selm[kIt], keepm[kIt];
-    uint2 rdj[kIt];
-#pragma unroll
-    for (int j = 0; j < kIt; ++j) {
-      selm[j] = keepm[j] = 0;
-      rdj[j] = make_uint2(0, 0);
-      const uint32_t base = warp * 32 + j * nthr;
-      if (base < nF) {
-        const uint32_t i = base + lane;
-        const bool valid = i < nF;
-        bool sel = false;
-        if (valid) {
-          const unsigned long long dv = r[j].d;
-          if (md.use_in) {
-            const uint32_t im = r[j].im;
-            sel = (im == kInf32) || dv <= minD + im;
-          }
-          if (!sel && md.use_out) sel = dv <= minOut;
-          const uint32_t v = sq[i];
-          if (sel) {
-            if (status_live(md, kNF)) w.status[v] = kS;
-            w.vrec[v].d = dv | kSettledBit;
-            if (w.settle_phase) w.settle_phase[v] = (uint32_t)k;
-            rdj[j] = __ldg(&g.rowdeg[v]);
-          } else {
-            pd = dv < pd ? dv : pd;
-            const uint32_t om = r[j].om;
-            if (om != kInf32) {
-              const unsigned long long x = dv + om;
-              po = x < po ? x : po;
-            }
-          }
+    since_pick = policy ? (since_pick + 1) & 7u : 1u;
+    const bool in_dyn = kKind != kStatic && arm.in_simple && use_in && w.cur_in != nullptr;
+    if (scribe && trace) s_t0 = globaltimer_ns();
+    live = m.used[tid] & ~spent;
+    if (SSSP_RARE(in_dyn || was_dyn)) {  // minima of this phase's variant (IN-SIMPLE reads status bytes the selection writes)
+      // (the warp's slots in use, dealt to its lanes evenly: a cursor's round
+      // trips follow one another)
+      uint8_t* ids = reinterpret_cast<uint8_t*>(m.list);
+      static_assert(8 * 32 <= 256 && kSoloList * sizeof(uint4) >= 8 * 32, "eight slots a thread at a time");
+      for (uint32_t j0 = 0; j0 < spt; j0 += 8) {
+        uint32_t n = 0;
+        for (uint32_t j = 0; j < min(spt - j0, 8u); ++j) {
+          const bool on = (live >> (j0 + j)) & 1u;
+          const unsigned int bm = __ballot_sync(0xFFFFFFFFu, on);
+          if (on) ids[n + __popc(bm & ((1u << lane) - 1u))] = (uint8_t)(j * 32 + lane);
+          n += __popc(bm);
         }
-        selm[j] = __ballot_sync(0xFFFFFFFFu, sel);
-        keepm[j] = __ballot_sync(0xFFFFFFFFu, valid && !sel);
-      }
-    }
-    uint32_t wk = 0, wr = 0, we = 0, ws = 0;
-#pragma unroll
-    for (int j = 0; j < kIt; ++j) {
-      if (warp * 32 + j * nthr >= nF) break;  // (warp-uniform) the rest of the steps are empty
-      const bool rl = ((selm[j] >> lane) & 1u) && rdj[j].y > 0;
-      wk += __popc(keepm[j]);
-      ws += __popc(selm[j]);
-      wr += __popc(__ballot_sync(0xFFFFFFFFu, rl));
-      we += __reduce_add_sync(0xFFFFFFFFu, rl ? rdj[j].y : 0u);
-    }
-    if (lane == 0) {
-      s_wk[warp] = wk;
-      s_wr[warp] = wr;
-      s_we[warp] = we;
-      if (ws) atomicAdd(&s_settled[pb], ws);
-    }
-    pd = warp_min_u64(pd);
-    po = warp_min_u64(po);
-    if (lane == 0) {
-      if (pd != kInf64) atomicMin(&s_thr_d[pb], pd);
-      if (po != kInf64 && md.use_out) atomicMin(&s_thr_o[pb], po);
-    }
-    __syncthreads();
-    if (tid == 0) {  // the next phase's counters (every thread has read them as the last phase's)
-      s_qn[pb ^ 1] = 0;
-      s_settled[pb ^ 1] = 0;
-      s_relax[pb ^ 1] = 0;
-      s_thr_d[pb ^ 1] = s_thr_o[pb ^ 1] = kInf64;
-      s_dfar[pb ^ 1] = 0;
-    }
-    {
-      // every warp scans the per-warp counts itself: its offsets and the totals
-      const unsigned int nw = nthr >> 5;
-      const uint32_t a = lane < nw ? s_wk[lane] : 0, b = lane < nw ? s_wr[lane] : 0, c = lane < nw ? s_we[lane] : 0;
-      const uint32_t ia = warp_inclusive_scan(a), ib = warp_inclusive_scan(b), ic = warp_inclusive_scan(c);
-      uint32_t koff = __shfl_sync(0xFFFFFFFFu, ia - a, warp);
-      uint32_t roff = __shfl_sync(0xFFFFFFFFu, ib - b, warp);
-      uint32_t eoff = __shfl_sync(0xFFFFFFFFu, ic - c, warp);
-      if (warp == 0 && lane == 31) {
-        s_qn[pb] = ia;
-        s_relax[pb] = ((unsigned long long)ib << 32) | ic;
-      }
-      const unsigned int lt = (1u << lane) - 1u;
-#pragma unroll
-      for (int j = 0; j < kIt; ++j) {
-        const uint32_t base = warp * 32 + j * nthr;
-        if (base < nF) {
-          const uint32_t i = base + lane;
-          if ((keepm[j] >> lane) & 1u) {
-            const uint32_t slot = koff + __popc(keepm[j] & lt);
-            const uint32_t v = sq[i];
-            if (slot < kSoloCap) sqn[slot] = v;
-            else if (slot < n) gqn[slot] = v;
-            else atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
-          }
-          koff += __popc(keepm[j]);
-          const bool rl = ((selm[j] >> lane) & 1u) && rdj[j].y > 0;
-          const unsigned int rm = __ballot_sync(0xFFFFFFFFu, rl);
-          const uint32_t c = rl ? rdj[j].y : 0u;
-          const uint32_t incl = warp_inclusive_scan(c);
-          if (rl) {
-            const uint32_t slot = roff + __popc(rm & lt);  // < |S'| <= nF <= kSoloCap
-            sp_d[slot] = r[j].d;
-            sp_row[slot] = rdj[j].x;
-            sp_base[slot] = eoff + incl - c;
-          }
-          roff += __popc(rm);
-          eoff += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        __syncwarp();
+        for (uint32_t i = lane; i < n; i += 32) {
+          const uint32_t s = (j0 + (ids[i] >> 5)) * nthr + warp * 32 + (ids[i] & 31u), v = m.slot[s].w;
+          m.slot[s].y = in_dyn ? in_min_dynamic(p.g, w, v, false) : __ldg(&p.g.in_min[v]);
         }
+        __syncwarp();
       }
-    }
-    __syncthreads();
-    const unsigned long long packed = s_relax[pb];
-    const uint32_t nS = (uint32_t)(packed >> 32), E = (uint32_t)packed;
-    if (can_handoff && E > p.solo_edges) {
-      // state of a grid selection step of phase k, in global memory
-      for (uint32_t j = tid; j < nS; j += nthr) {
-        *reinterpret_cast<ulonglong2*>(&w.sp[j]) =
-            make_ulonglong2(sp_d[j], (unsigned long long)sp_row[j] | ((unsigned long long)sp_base[j] << 32));
-        if (w.tile_owner) mark_tile_owner(w.tile_owner, j, sp_base[j], (j + 1 < nS ? sp_base[j + 1] : E) - sp_base[j]);
-      }
-      const uint32_t kept = s_qn[pb];
-      const uint32_t nk = kept < kSoloCap ? kept : kSoloCap;
-      for (uint32_t j = tid; j < nk; j += nthr) gqn[j] = sqn[j];
-      if (tid == 0) {
-        st.sum_f += fs;
-        ctl->far_count = far;
-        PhaseSlot* S0 = &ctl->slot[k % 4];
-        PhaseSlot* S1 = &ctl->slot[(k + 1) % 4];
-        reset_slot(S0);
-        reset_slot(S1);
-        reset_slot(&ctl->slot[(k + 2) % 4]);
-        S0->qcount = nF;
-        S0->fsize = fs;
-        S0->min_d = minD;
-        S0->min_out = minOut;
-        S0->relax_packed = packed;
-        S0->settled_now = s_settled[pb];
-        S0->arm = arm_code(arm, true) | nf_code;
-        S0->t_start = s_t0;
-        S0->t_select = globaltimer_ns();
-        S1->qcount = kept;
-        S1->min_d = s_thr_d[pb];
-        S1->min_out = s_thr_o[pb];
-      }
-      __threadfence();
+      was_dyn = in_dyn;
       __syncthreads();
-      *handoff = true;
-      return k;
     }
-    // ---- C: relax
-    if (tid == 0 && w.trace) s_tsel = globaltimer_ns();
-    pd = kInf64;
-    po = kInf64;
-    int dfar = 0;
-    const SoloRelax sr{sp_d, sp_row, sp_base, nS, E, sqn, gqn, &s_qn[pb]};
-    if (kNF) solo_relax<true>(p, md, sr, nv, pd, po, dfar);
-    else solo_relax<false>(p, md, sr, nv, pd, po, dfar);
-    pd = warp_min_u64(pd);
-    po = warp_min_u64(po);
-    if (kNF) dfar = __reduce_add_sync(0xFFFFFFFFu, dfar);
-    if (lane == 0) {
-      if (pd != kInf64) atomicMin(&s_thr_d[pb], pd);
-      if (po != kInf64 && md.use_out) atomicMin(&s_thr_o[pb], po);
-      if (dfar) atomicAdd(&s_dfar[pb], dfar);
+    if (kNarrow && SSSP_RARE(minD > kSoloRebase)) {
+      for (uint32_t b = live; b; b &= b - 1) *m.d((uint32_t)(__ffs(b) - 1) * nthr + tid) -= minD;
+      base += minD;
+      if (minOut != inf) minOut -= minD;
+      minD = 0;
     }
-    __syncthreads();
-    const uint32_t nFn = s_qn[pb];
-    const uint32_t settled_now = s_settled[pb];
-    if (tid == 0) {
-      st.phases = k;
-      st.sum_f += fs;
-      st.settled += settled_now;
-      st.relaxed += E;
-      ctl->heartbeat = k;
-      if (w.trace && k <= w.trace_cap) {
-        sssp_phase_record r;
-        r.frontier = fs;
-        r.settled = settled_now;
-        r.min_d = minD;
-        r.min_out = md.use_out ? minOut : kInf64;
-        r.deg_settled = E;
-        uint32_t c = p.crit & SSSP_CRITERIA_MASK;
-        if (md.use_in) c = (c & ~(uint32_t)(SSSP_IN_STATIC | SSSP_IN_SIMPLE)) | (in_dyn ? SSSP_IN_SIMPLE : SSSP_IN_STATIC);
-        r.criterion = c;
-        r.arm = arm_code(arm, true) | nf_code;
-        r.t_start_ns = s_t0;
-        r.t_end_ns = globaltimer_ns();
-        r.queued = nF;
-        r.select_ns = (uint32_t)(s_tsel - s_t0);
-        w.trace[k - 1] = r;
+    // ---- select
+    od = oo = inf;
+    sel = 0;
+    for (uint32_t j0 = 0; j0 < spt; j0 += 4) {
+      if (!__any_sync(0xFFFFFFFFu, (live | spent) >> j0)) break;
+      uint4 q[4];
+      T d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t s = (j0 + u) * nthr + tid;
+        q[u] = m.slot[s];
+        d[u] = kNarrow ? (T)q[u].x : *m.d(s);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t bit = 1u << (j0 + u), s = (j0 + u) * nthr + tid;
+        const bool lv = (live & bit) != 0;
+        const bool in = (d[u] - minD <= q[u].y) | (!kNarrow & (q[u].y == kInf32));
+        const bool is = lv & ((use_in & in) | (use_out & (d[u] <= minOut)));
+        const T x = q[u].z != kInf32 ? d[u] + q[u].z : inf;
+        const T kd = lv & !is ? d[u] : inf, ko = lv & !is ? x : inf;
+        od = kd < od ? kd : od;
+        oo = ko < oo ? ko : oo;
+        if (spent & bit) *m.d(s) = inf;
+        sel |= is ? bit : 0u;
       }
     }
-    nf_code &= ~(kArmNfRefill | kArmNfPull);  // a refill, pull or split only runs before the episode
-    minD = s_thr_d[pb];
-    minOut = s_thr_o[pb];
+    // mark and list the settled vertices
+    uint32_t nsel = 0, deg = 0;  // vertices settled by the warp; edges of this thread's
+    {
+      uint32_t rest = sel;
+      for (unsigned int bm; (bm = __ballot_sync(0xFFFFFFFFu, rest != 0)) != 0;) {
+        if (rest) {
+          const uint32_t s = (uint32_t)(__ffs(rest) - 1) * nthr + tid;
+          const uint32_t at = nsel + __popc(bm & ((1u << lane) - 1u));
+          const uint2 row = m.row[s];
+          const uint32_t v = m.slot[s].w;
+          const T dv = *m.d(s);
+          rest &= rest - 1;
+          deg += min(row.y, 0xFFFFu);
+          if (at < kSoloList)
+            m.list[at] = make_uint4(row.x, row.y, (uint32_t)dv, (uint32_t)((unsigned long long)dv >> 32));
+          vrec[v].d = (base + dv) | kSettledBit;
+          if (kKind != kStatic && status) status[v] = kS;
+          if (settle) w.settle_phase[v] = k;
+          if (kNarrow && dv > kSoloLastD) sc->stop = 1;
+        }
+        nsel += __popc(bm);
+      }
+    }
+    m.used[tid] = live;  // (with the slots just settled: their D is needed for a hand-off)
+    spent = sel;
+    // Slots for new vertices: those of warp (warp + k) % nw, whose mask is read
+    // while that warp may be freeing some (an older mask has more in use) and
+    // again after the barrier.
+    const uint32_t owner = (((warp + k) & (nw - 1)) << 5) + lane, full = (1u << spt) - 1u;
+    uint32_t free = ~*reinterpret_cast<volatile uint32_t*>(&m.used[owner]) & full;
+    // Deals the next edges to the lanes with a free slot (one among the first
+    // four if there are enough of them, from another lane on in every phase: so
+    // the lanes' slots fill alike, the first four before the rest) and issues
+    // their loads.  `q`: this lane's entry of the warp's list, with {out-row
+    // start less the degrees before it, degrees up to and with it} for its row;
+    // `pos`: edges dealt.  A heavy phase deals out the edges [pos, end) of the
+    // whole block's lists instead (`wc`: lane j has warp j's edges, settled
+    // vertices and the edges up to and with it).
+    const uint32_t turn = (k * 11u) & 31u;
+    uint32_t left = 0, pos = 0, end = 0;
+    unsigned int fm = 0;
+    uint4 q = make_uint4(0, 0, 0, 0);
+    uint3 wc = make_uint3(0, 0, 0);
+    uint2 ed = make_uint2(0, 0);
+    T src = 0;
+    bool act = false, heavy = false;
+    auto deal = [&]() {
+      const uint32_t want = min(end - pos, 32u);
+      bool mine = (free & 15u) != 0;
+      fm = __ballot_sync(0xFFFFFFFFu, mine);
+      if (__popc(fm) < want) {
+        mine = free != 0;
+        fm = __ballot_sync(0xFFFFFFFFu, mine);
+      }
+      const uint32_t take = min(want, (uint32_t)__popc(fm));
+      const uint32_t rank = __popc(__funnelshift_r(fm, fm, turn) & ((1u << ((lane - turn) & 31u)) - 1u));
+      const uint32_t e = pos + min(rank, take - 1);
+      uint32_t at;
+      if (!heavy) {
+        uint32_t l = 0;  // lane whose row holds edge e
+#pragma unroll
+        for (uint32_t step = 16; step > 0; step >>= 1)
+          if (__shfl_sync(0xFFFFFFFFu, q.y, l + step - 1) <= e) l += step;
+        at = __shfl_sync(0xFFFFFFFFu, q.x, l) + e;
+        src = (T)__shfl_sync(0xFFFFFFFFu, q.z, l);
+        if (!kNarrow) src |= (T)((unsigned long long)__shfl_sync(0xFFFFFFFFu, q.w, l) << 32);
+      } else {
+        uint32_t l = 0;  // warp whose list holds edge e
+        for (uint32_t step = nw >> 1; step > 0; step >>= 1)
+          if (__shfl_sync(0xFFFFFFFFu, wc.z, l + step - 1) <= e) l += step;
+        const uint32_t el = e - (__shfl_sync(0xFFFFFFFFu, wc.z, l) - __shfl_sync(0xFFFFFFFFu, wc.x, l));
+        const uint4* list = m.list + ((int)l - (int)warp) * (int)kSoloList;
+        uint32_t a = 0, b = __shfl_sync(0xFFFFFFFFu, wc.y, l) - 1;  // its first entry with more edges than el before its end
+        while (a < b) {
+          const uint32_t mid = (a + b) >> 1;
+          if (list[mid].y <= el) a = mid + 1; else b = mid;
+        }
+        const uint4 t = list[a];
+        at = t.x + el;
+        src = kNarrow ? (T)t.z : (T)(t.z | ((unsigned long long)t.w << 32));
+      }
+      act = mine && rank < take;
+      if (act) ed = __ldg(&edges[at]);
+      pos += take;
+    };
+    const uint32_t room = __reduce_add_sync(0xFFFFFFFFu, __popc(free));
+    if (nsel > 0) {
+      __syncwarp();  // (the list)
+      left = __reduce_add_sync(0xFFFFFFFFu, deg);
+      if (lane < min(nsel, kSoloList)) q = m.list[lane];
+      const uint32_t incl = warp_inclusive_scan(q.y);
+      q.x -= incl - q.y;
+      q.y = incl;
+      if (lane == 0) {
+        atomicAdd(&sc->settled, nsel);
+        atomicAdd(&sc->edges, left);
+        if (left > kSoloHeavy || left > room) sc->heavy = 1;
+        if (nsel > kSoloList) sc->stop = 1;
+      }
+      end = left;
+      if (left > 0 && left <= kSoloHeavy && left <= room && nsel <= kSoloList) deal();
+    }
+    if (lane == 0) atomicMin(&sc->room, room);
+    __syncthreads();
+    const uint32_t E = sc->edges;
+    if (scribe && trace) s_tsel = globaltimer_ns();
+    const uint32_t settled_now = sc->settled;
+    heavy = sc->heavy != 0;
+    if (SSSP_RARE(E > p.solo_edges || sc->stop || (heavy && E > nw * min(sc->room, 0x10000u)))) {
+      hand = true;
+      break;
+    }
+    if (tid < sizeof(SoloCount) / 4)  // the next phase's counters (solo_clear, word by word)
+      reinterpret_cast<uint32_t*>(&s_sc[(k + 1) & 1])[tid] = (tid >= 4 && tid < 8) || tid == 10 ? kInf32 : 0u;
+    // ---- relax
+    int nfar = 0;
+    uint32_t nnew = 0;
+    uint32_t used = m.used[owner];
+    if (SSSP_RARE(heavy)) {  // (what the light deal has loaded is in the L1 cache now)
+      if (lane < nsel) m.list[lane] = q;
+      if (lane == 0) s_warp[warp] = make_uint2(left, nsel);
+      __syncthreads();
+      const uint2 c = lane < nw ? s_warp[lane] : make_uint2(0, 0);
+      wc = make_uint3(c.x, c.y, warp_inclusive_scan(c.x));
+      const uint32_t run = (E + nw - 1) >> (31 - __clz(nw));
+      pos = min(warp * run, E);
+      end = min(pos + run, E);
+      free = ~used & full;
+      fm = 0;
+      if (pos < end) deal();
+    }
+    while (fm) {
+      const uint32_t s = (uint32_t)(__ffs(~used) - 1) * nthr + owner;  // the slot for a new vertex
+      const uint32_t t = ed.x;
+      bool claimed = false;
+      uint32_t app = kNoBucket;
+      if (act) {
+        const T cand = src + ed.y;
+        unsigned long long x;  // what t's word holds, once known: a slot number if t is in the near fringe
+        uint32_t im, om;
+        uint2 trow = make_uint2(0, 0);
+        bool lowered = true;
+        if (!kNF) {
+          x = atomicCAS(&vrec[t].d, kUnexplored, (unsigned long long)s);
+          const uint2 mm = __ldcg(reinterpret_cast<const uint2*>(&vrec[t].im));
+          trow = __ldg(&rowdeg[t]);
+          im = mm.x;
+          om = mm.y;
+          claimed = x == kUnexplored;
+          lowered = !(x & kSettledBit);
+          if (kKind != kStatic && claimed && status) status[t] = kF;
+          x = claimed ? s : x;
+        } else {
+          const VRec r = ldcg_vrec(&vrec[t]);
+          x = r.d;
+          im = r.im;
+          om = r.om;
+          const unsigned long long c64 = base + cand;
+          if (x >= kFarBit && !(x & kSettledBit) && c64 > nv.bound + im) {
+            // unexplored or far, and far with this candidate (a slot number,
+            // should another relaxation claim t now, is lower and stays)
+            const unsigned long long enc = c64 | kFarBit;
+            lowered = false;
+            if (enc < x) {
+              x = atomicMin(&vrec[t].d, enc);
+              lowered = enc < x;
+              if (x == kUnexplored) {
+                ++nfar;
+                if (kKind != kStatic && status) status[t] = kF;
+                if (nv.lists) app = nf_bucket(nv, enc, im);
+              } else if (lowered && nv.lists) {
+                const uint32_t b = nf_bucket(nv, enc, im);
+                if (b != nf_bucket(nv, x, im)) app = b;
+              }
+            }
+            x = kSettledBit;  // (no slot to lower)
+          } else {
+            while (x >= kFarBit && !(x & kSettledBit)) {  // claim it (a far vertex may be lowered meanwhile: again)
+              const unsigned long long o = atomicCAS(&vrec[t].d, x, (unsigned long long)s);
+              if (o == x) {
+                claimed = true;
+                if (x != kUnexplored) --nfar;
+                else if (kKind != kStatic && status) status[t] = kF;
+                trow = __ldg(&rowdeg[t]);
+                x = s;
+              } else {
+                x = o;
+              }
+            }
+            lowered = !(x & kSettledBit);
+          }
+        }
+        if (claimed) {
+          m.slot[s].y = im;
+          m.slot[s].z = om;
+          m.slot[s].w = t;
+          m.row[s] = trow;
+          used |= ~used & (used + 1);
+        }
+        if (!(x & kSettledBit)) atomicMin(m.d((uint32_t)x), cand);
+        if (lowered) {
+          od = cand < od ? cand : od;
+          const T c2 = om != kInf32 ? cand + om : inf;
+          oo = c2 < oo ? c2 : oo;
+        }
+      }
+      if (kNF) nf_list_append(nv, app, t);
+      nnew += __popc(__ballot_sync(0xFFFFFFFFu, claimed));
+      if (pos == end) break;
+      free = ~used & full;
+      deal();
+    }
+    if (nnew) {
+      m.used[owner] = used;
+      if (lane == 0) atomicAdd(&sc->fresh, nnew);
+    }
+    if (kNF) {
+      const int df = __reduce_add_sync(0xFFFFFFFFu, nfar);
+      if (lane == 0 && df) atomicAdd(&sc->far, df);
+    }
+    od = solo_warp_min(od);
+    oo = solo_warp_min(oo);
+    if (lane == 0) {
+      atomicMin(solo_thr<T>(&sc->min_d), od);
+      atomicMin(solo_thr<T>(&sc->min_out), oo);
+    }
+    __syncthreads();
+    const uint32_t fs = nF + far;  // |F| at the start of the phase
+    sum_f += fs;
+    sum_s += settled_now;
+    sum_e += E;
     e_prev = E;
     s_prev = settled_now;
     f_prev = fs;
-    nF = nFn;
-    if (kNF) far += (uint32_t)s_dfar[pb];
+    if (tid == 0) ctl->heartbeat = k;
+    if (trace && scribe && k <= w.trace_cap) {
+      sssp_phase_record r;
+      r.frontier = fs;
+      r.settled = settled_now;
+      r.min_d = base + minD;
+      r.min_out = use_out && minOut != inf ? base + minOut : kInf64;
+      r.deg_settled = E;
+      uint32_t c = p.crit & SSSP_CRITERIA_MASK;
+      if (use_in) c = (c & ~(uint32_t)(SSSP_IN_STATIC | SSSP_IN_SIMPLE)) | (in_dyn ? SSSP_IN_SIMPLE : SSSP_IN_STATIC);
+      r.criterion = c;
+      r.arm = arm_code(arm, true) | nf_code;
+      r.t_start_ns = s_t0;
+      r.t_end_ns = globaltimer_ns();
+      r.queued = nF;
+      r.select_ns = (uint32_t)(s_tsel - s_t0);
+      w.trace[k - 1] = r;
+    }
+    nf_code &= ~(kArmNfRefill | kArmNfPull);  // a refill, pull or split only runs before the episode
+    nF = nF - settled_now + sc->fresh;
+    if (kNF) far += (uint32_t)sc->far;
+    minD = *solo_thr<T>(&sc->min_d);
+    minOut = use_out ? *solo_thr<T>(&sc->min_out) : inf;
     ++k;
-    if (nF == 0 || nF > cap || k > (uint64_t)n + 1) break;
+    if (nF == 0 || nF > solo_stay(p) || k > p.g.n + 1) break;
     // thresholds above the bound are exact only after the far part is scanned
-    if (kNF && far > 0 && (md.use_out ? minOut : minD) > nv.bound) break;
+    if (kNF && far > 0) {
+      const T x = use_out ? minOut : minD;
+      if (x == inf || base + x > nv.bound) break;
+    }
+  }
+  if (tid == 0) {
+    if (sum_s > 0) s_st.phases = k - 1;
+    s_st.sum_f += sum_f;
+    s_st.settled += sum_s;
+    s_st.relaxed += sum_e;
+  }
+  if (hand) {
+    if (tid == 0) s_solo_arm = arm;
+    solo_hand_off<T>(k, live & ~sel, sel, od, oo, base, minD, minOut, nF, far, nf_code, s_t0);
+    if (tid == 0 && (!group || (uint32_t)s_solo_n <= p.solo_edges)) {
+      s_solo_cont = 1;
+      s_solo_since = since_pick;
+    }
+    __threadfence();
+    __syncthreads();
+    return 4ull * k + kSoloResume;
   }
   // hand the state back in global memory for phase k
-  {
-    const uint32_t* sq = ((k - 1) & 1) ? sqb : sqa;
-    uint32_t* gq = w.q[(k - 1) & 1];
-    const uint32_t ns = nF < kSoloCap ? nF : kSoloCap;
-    for (uint32_t i = tid; i < ns; i += nthr) gq[i] = sq[i];
-  }
+  if (tid == 0) s_solo_n = 0;
+  __syncthreads();
+  solo_write_back(m, m.used[tid] & ~spent, base, w.q[(k - 1) & 1]);
   if (tid == 0) {
     PhaseSlot* S0 = &ctl->slot[k % 4];
     reset_slot(S0);
     reset_slot(&ctl->slot[(k + 1) % 4]);
     ctl->far_count = far;
     S0->qcount = nF;
-    S0->min_d = minD;
-    S0->min_out = minOut;
+    if (minD != inf) S0->min_d = base + minD;
+    if (minOut != inf) S0->min_out = base + minOut;
     PhaseSlot* Sp = &ctl->slot[(k + 3) % 4];  // the last solo phase, for the policy's features
     Sp->relax_packed = e_prev;
-    Sp->settled_now = (uint32_t)s_prev;
-    Sp->fsize = (uint32_t)f_prev;
+    Sp->settled_now = s_prev;
+    Sp->fsize = f_prev;
   }
   __threadfence();
   __syncthreads();
-  return k;
+  return 4ull * k;
 }
 
 // ---------------------------------------------------------------------------
@@ -1615,11 +1946,18 @@ __device__ __forceinline__ void nf_lists_reset(const Grp& grp, Ctl* ctl) {
 // exact): B = T + the key offset below which about `target` queue entries lie;
 // entries above B are marked far and the queue is compacted.  Leaves B as is
 // when the whole fringe fits the target.  Every block of the group calls it.
-__device__ __noinline__ bool nf_split(const SolveParams& p, const Grp& grp, const Mode& md, uint64_t k, const Shared& sh,
-                                      NfView& nv, uint32_t& uses) {
+// Returns kNfFail if a barrier gave up, kNfUsed if it used a histogram, else kNfIdle.
+enum { kNfFail = 0, kNfIdle, kNfUsed };
+
+__device__ __noinline__ int nf_split(uint64_t k, uint32_t uses) {
+  const SolveParams& p = s_p;
+  const Grp& grp = s_grp;
+  const Mode& md = s_md;
+  NfView& nv = s_nv;
+  const Shared sh = carve();
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr();
   const uint64_t gthreads = (uint64_t)grp.size * nthr;
   const uint64_t gtid = (uint64_t)grp.rank * nthr + tid;
   const bool leader = grp.rank == 0 && tid == 0;
@@ -1627,7 +1965,7 @@ __device__ __noinline__ bool nf_split(const SolveParams& p, const Grp& grp, cons
   uint32_t* Q = w.q[(k - 1) & 1];
   const uint32_t nF = ldcg_u32(&S0->qcount);
   const unsigned long long T = md.use_out ? ldcg_u64(&S0->min_out) : ldcg_u64(&S0->min_d);
-  if (T >= kNoBound) return true;
+  if (T >= kNoBound) return kNfIdle;
   unsigned int* gh = ctl->hist[uses & 1];
   uint32_t* hist = sh.s_base;
   nf_hist_clear(hist);
@@ -1645,13 +1983,12 @@ __device__ __noinline__ bool nf_split(const SolveParams& p, const Grp& grp, cons
   if (leader) ctl->nf_tmp = 0;
   if (tid < kNfBins && grp.rank == 0) ctl->hist[(uses + 1) & 1][tid] = 0;  // the next use's histogram
   nf_lists_reset(grp, ctl);
-  ++uses;
-  if (!grp.sync()) return false;
+  if (!grp.sync()) return kNfFail;
   const int b = nf_pick_bin(gh, nf_target(p, k, nF), sh);
-  if (b >= kNfBins) return true;
+  if (b >= kNfBins) return kNfUsed;
   const unsigned long long e = nf_bin_upper(b);
   const unsigned long long B = e >= kNoBound - T ? kNoBound : T + e;
-  if (B >= kNoBound) return true;
+  if (B >= kNoBound) return kNfUsed;
   const NfView v2 = nf_geometry(nv, B, e);
   // keep the entries with key <= B (compacted into the relax-list buffer),
   // mark the others far and list them in their buckets
@@ -1682,12 +2019,12 @@ __device__ __noinline__ bool nf_split(const SolveParams& p, const Grp& grp, cons
   uint32_t td;
   block_exclusive_scan(demoted, sh.scan, &td);
   if (tid == 0 && td) atomicAdd(&ctl->far_count, td);
-  if (!grp.sync()) return false;
+  if (!grp.sync()) return kNfFail;
   const uint32_t kept = ldcg_u32(&ctl->nf_tmp);
   for (uint64_t i = gtid; i < kept; i += gthreads) Q[i] = ldcg_u32(&tmp[i]);
   if (leader) S0->qcount = kept;
   if (tid == 0) nv = v2;  // (published to the block by the barrier below)
-  return grp.sync();
+  return grp.sync() ? kNfUsed : kNfFail;
 }
 
 // Refill (far part not empty, accumulated T > B).  R1: every block scans its
@@ -1701,13 +2038,17 @@ __device__ __noinline__ bool nf_split(const SolveParams& p, const Grp& grp, cons
 // of the group calls it.
 constexpr int kNfItems = 8;
 
-__device__ __noinline__ bool nf_refill(const SolveParams& p, const Grp& grp, const Mode& md, uint64_t k, const Shared& sh,
-                                       NfView& nv, uint32_t& uses) {
+__device__ __noinline__ bool nf_refill(uint64_t k, uint32_t uses) {
+  const SolveParams& p = s_p;
+  const Grp& grp = s_grp;
+  const Mode& md = s_md;
+  NfView& nv = s_nv;
+  const Shared sh = carve();
   const GraphView& g = p.g;
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
   const uint32_t n = g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr(), lane = tid & 31;
   const bool leader = grp.rank == 0 && tid == 0;
   PhaseSlot* S0 = &ctl->slot[k % 4];
   uint32_t* Q = w.q[(k - 1) & 1];
@@ -1768,7 +2109,6 @@ __device__ __noinline__ bool nf_refill(const SolveParams& p, const Grp& grp, con
   nf_hist_flush(hist, gh);
   if (tid < kNfBins && grp.rank == 0) ctl->hist[(uses + 1) & 1][tid] = 0;
   nf_lists_reset(grp, ctl);
-  ++uses;
   if (!grp.sync()) return false;
   const unsigned long long a_d = ldcg_u64(&S0->min_d), f_d = ldcg_u64(&S0->a_min_d);
   const unsigned long long a_o = ldcg_u64(&S0->min_out), f_o = ldcg_u64(&S0->a_min_out);
@@ -1838,16 +2178,21 @@ __device__ __noinline__ bool nf_refill(const SolveParams& p, const Grp& grp, con
 // clears the far bit moves it; stale and duplicate entries are skipped),
 // taking the minima of d and d + outmin over the moved vertices into the
 // phase's thresholds.  The vertex attaining T is among them or in the queue,
-// every far vertex left has key > B' >= T, so the thresholds stay exact.  Sets
-// *need_full (and changes nothing) when a full refill is needed instead: the
+// every far vertex left has key > B' >= T, so the thresholds stay exact.  Returns
+// kNfIdle (and changes nothing) when a full refill is needed instead: the
 // bucket holding T lies past the ring or at or after the lowest bucket with an
-// unlisted vertex.  Every block of the group calls it.
-__device__ __noinline__ bool nf_pull(const SolveParams& p, const Grp& grp, const Mode& md, uint64_t k, const Shared& sh,
-                                     NfView& nv, bool* need_full) {
+// unlisted vertex; kNfUsed after a pull, kNfFail if a barrier gave up.  Every
+// block of the group calls it.
+__device__ __noinline__ int nf_pull(uint64_t k) {
+  const SolveParams& p = s_p;
+  const Grp& grp = s_grp;
+  const Mode& md = s_md;
+  NfView& nv = s_nv;
+  const Shared sh = carve();
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
   const uint32_t n = p.g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr(), lane = tid & 31, warp = tid >> 5;
   PhaseSlot* S0 = &ctl->slot[k % 4];
   uint32_t* Q = w.q[(k - 1) & 1];
   __shared__ uint32_t s_pre[kNfRing + 1];
@@ -1888,8 +2233,7 @@ __device__ __noinline__ bool nf_pull(const SolveParams& p, const Grp& grp, const
   __syncthreads();
   const uint32_t nb = s_nb;
   if (nb == 0) {
-    *need_full = true;
-    return true;
+    return kNfIdle;
   }
   const unsigned long long B1 = s_newb;
   const uint32_t total = s_pre[nb];
@@ -1940,7 +2284,7 @@ __device__ __noinline__ bool nf_pull(const SolveParams& p, const Grp& grp, const
   // the selection step takes min(min_d, a_min_d) and min(min_out, a_min_out)
   block_min2_to_global(lmin_d, lmin_o, &S0->a_min_d, md.use_out ? &S0->a_min_out : nullptr, sh.red);
   if (lane == 0 && moved) atomicAdd(&ctl->nf_moved, moved);
-  if (!grp.sync()) return false;
+  if (!grp.sync()) return kNfFail;
   if (grp.rank == 0) {
     // the pulled slots start over as the buckets past the ring's far end (no
     // block lists a far vertex before the next selection step's barrier)
@@ -1956,47 +2300,28 @@ __device__ __noinline__ bool nf_pull(const SolveParams& p, const Grp& grp, const
     nv.cursor = c + nb;
   }
   __syncthreads();
-  return true;
+  return kNfUsed;
 }
 
-// Initialise, run all phases (switching to solo mode while the fringe is
-// small), write the distances.  Every block of the group calls it.
-// `p` is the block's shared copy of the parameters (what the out-of-line
-// phase steps take); `pk` is the same parameters where the inlined solo
-// episodes read them fastest (the kernel parameter bank of a single solve).
-__device__ void solve_body(const SolveParams& p, const SolveParams& pk, const Grp& grp_in, unsigned char* smem) {
+// The parts of a solve (initialise, grid phases, solo episodes, write the
+// distances) are apart, so that what one of them keeps in registers is not held
+// through the others.  Every block of the group calls them; false: a barrier
+// gave up.
+__device__ __noinline__ bool solve_init(const Grp grp_in) {
+  const SolveParams& p = s_p;
   const GraphView& g = p.g;
   const SolveWS& w = p.ws;
   Ctl* ctl = w.ctl;
   const uint32_t n = g.n;
-  const unsigned int tid = threadIdx.x, nthr = blockDim.x;
-  // The group, the shared-memory layout and the mode are the same for every
-  // thread of the block: one copy in shared memory, which the steps read
-  // through references (per-thread copies would live in local memory).
-  __shared__ Grp s_grp;
-  __shared__ Shared s_sh;
-  __shared__ Mode s_md;
+  const unsigned int tid = opaque_tid(), nthr = opaque_nthr();
   if (tid == 0) {
     s_grp = grp_in;
-    s_sh = carve(smem);
+    s_grp1 = Grp{grp_in.bar, grp_in.err, grp_in.limit, 0, 1};
     s_md = mode_of(p);
-  }
-  __syncthreads();
-  const Grp& grp = s_grp;
-  const Shared& sh = s_sh;
-  const Mode& md = s_md;
-  const uint64_t gthreads = (uint64_t)grp.size * nthr;
-  const uint64_t gtid = (uint64_t)grp.rank * nthr + tid;
-  const bool leader = grp.rank == 0 && tid == 0;
-  // Counters and the near/far bound live in shared memory: they are touched
-  // once per phase at most, and keeping them out of registers leaves the
-  // phase loops more room.
-  __shared__ Stats s_st;
-  __shared__ NfView s_nv;  // near/far bound and bucket geometry (same in every block)
-  Stats& st = s_st;
-  if (tid == 0) {
     s_st = Stats{0, 0, 0, 0};
     s_arm_k = ~0ull;
+    s_solo_cont = 0;
+    s_nf_uses = 0;
     s_nv.bound = kNoBound;
     s_nv.origin = 0;
     s_nv.shift = 0;
@@ -2006,9 +2331,14 @@ __device__ void solve_body(const SolveParams& p, const SolveParams& pk, const Gr
     s_nv.cnt = ctl->nf_cnt;
     s_nv.beyond = &ctl->nf_beyond;
   }
+  __syncthreads();
+  const Grp& grp = s_grp;
+  const uint64_t gthreads = (uint64_t)grp.size * nthr;
+  const uint64_t gtid = (uint64_t)grp.rank * nthr + tid;
+  const bool leader = grp.rank == 0 && tid == 0;
   if ((p.crit & SSSP_POLICY_LEARNED) && p.policy) {  // (published by the first barrier below)
-    float* pw = reinterpret_cast<float*>(smem + kPolicySmemOffset);
-    for (int i = tid; i < kPolWeights; i += nthr) pw[i] = __ldg(&p.policy[i]);
+    float* pw = reinterpret_cast<float*>(smem_all + p.pol_off);
+    for (int i = tid; i < kPolWeights; i += nthr) pw[policy_place(i)] = __ldg(&p.policy[i]);
   }
 
   for (uint64_t v = gtid; v < n; v += gthreads) {
@@ -2032,13 +2362,12 @@ __device__ void solve_body(const SolveParams& p, const SolveParams& pk, const Gr
     for (int j = 0; j < 4; ++j) reset_slot(&ctl->slot[j]);
     ctl->heartbeat = 0;
     ctl->next_phase = 0;
-    ctl->resume_relax = 0;
     ctl->far_count = 0;
     ctl->nf_tmp = 0;
   }
   if (grp.rank == 0)
     for (int b = tid; b < 2 * kNfBins; b += nthr) ctl->hist[b / kNfBins][b % kNfBins] = 0;
-  if (!grp.sync()) return;
+  if (!grp.sync()) return false;
   if (leader) {
     w.vrec[p.source].d = 0;
     w.status[p.source] = kF;
@@ -2049,139 +2378,182 @@ __device__ void solve_body(const SolveParams& p, const SolveParams& pk, const Gr
     const uint32_t om = __ldg(&g.out_min[p.source]);
     s1->min_out = om == kInf32 ? kInf64 : (unsigned long long)om;
   }
-  if (!grp.sync()) return;
+  return grp.sync();
+}
 
-  const bool dense_forced = (p.crit & SSSP_FRONTIER_DENSE) != 0;
-  const uint32_t solo_cap = p.solo_max < kSoloCap ? p.solo_max : kSoloCap;
+// Solo phases of the three-step kind: the generic phase on this block alone.
+__device__ __noinline__ uint64_t generic_solo(uint64_t k) {
+  const SolveParams& p = s_p;
+  Ctl* const ctl = p.ws.ctl;
+  PhaseHead h = load_head(ctl, k, false);
+  while (h.nQ != 0 && h.nQ <= p.solo_max && k <= (uint64_t)p.g.n + 1) {
+    run_phase<kAny>(true, k, 0u, h);
+    ++k;
+    if (threadIdx.x == 0) ctl->heartbeat = k;
+    h = load_head(ctl, k, false);
+  }
+  return k;
+}
+
+// The leading block's word to the group after an episode, and the others' wait
+// for it (0 if the wait ran out): what solo_episode returned.
+__device__ __noinline__ void episode_end(uint64_t r) {
+  Ctl* const ctl = s_p.ws.ctl;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ctl->next_phase = r;
+    __threadfence();
+    red_release_gpu_add(&ctl->gate, 1u);
+  }
+  __syncthreads();
+}
+__device__ __noinline__ uint64_t episode_wait(unsigned int episodes) {
+  __shared__ unsigned long long s_next;
+  Ctl* const ctl = s_p.ws.ctl;
+  if (threadIdx.x == 0) {
+    const bool ok = bounded_wait_change(&ctl->gate, episodes, s_grp.limit, s_grp.err, &ctl->heartbeat);
+    s_next = ok ? ld_relaxed_gpu_u64(&ctl->next_phase) : 0ull;
+  }
+  __syncthreads();
+  const uint64_t r = s_next;
+  __syncthreads();
+  return r;
+}
+
+__device__ __noinline__ bool solve_finish() {
+  const SolveWS& w = s_p.ws;
+  const Grp& grp = s_grp;
+  const uint32_t n = s_p.g.n;
+  const uint64_t gthreads = (uint64_t)grp.size * blockDim.x;
+  const uint64_t gtid = (uint64_t)grp.rank * blockDim.x + threadIdx.x;
+  if (grp.rank == 0 && threadIdx.x == 0) {
+    w.ctl->phases = s_st.phases;
+    w.ctl->sum_f = s_st.sum_f;
+    w.ctl->settled = s_st.settled;
+    w.ctl->relaxed = s_st.relaxed;
+  }
+  if (!grp.sync()) return false;
+  for (uint64_t v = gtid; v < n; v += gthreads) {
+    const unsigned long long d = ldcg_u64(&w.vrec[v].d) & ~kSettledBit;
+    w.dist[v] = d == kUnexplored ? kInf64 : d;
+  }
+  return true;
+}
+
+// A whole solve: phases on the whole group, and episodes on one block while the
+// fringe is small.  The loop is part of the kernel: a function in between would
+// save and restore its caller's registers around every step once more.
+template <int kKind>
+__device__ __forceinline__ void solve_body(const Grp& grp_in) {
+  if (!solve_init(grp_in)) return;
+  const SolveParams& p = s_p;
+  const Grp& grp = s_grp;
+  const Mode& md = s_md;
+  const NfView& nv = s_nv;
   unsigned int episodes = 0;
-  NfView& nv = s_nv;
-  uint32_t nf_uses = 0;
-  uint64_t k = 1;
-  for (;;) {
+  bool forced = false;  // phase k by the group whatever its size
+  for (uint64_t k = 1;;) {
+    Ctl* const ctl = p.ws.ctl;
     PhaseHead h = load_head(ctl, k, nv.bound != kNoBound);
-    uint32_t nF = h.nQ;
     uint32_t nf_code = 0;
-    if (k > (uint64_t)n + 1) {  // every phase settles a vertex: more phases mean a broken invariant
-      if (leader) atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
+    if (SSSP_RARE(k > (uint64_t)p.g.n + 1)) {  // every phase settles a vertex: more phases mean a broken invariant
+      if (grp.rank == 0 && threadIdx.x == 0) atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
       break;
     }
     if (md.nearfar) {
-      const uint32_t far = h.far;
-      if (nF == 0 && far == 0) break;
+      if (h.nQ == 0 && h.far == 0) break;
       const unsigned long long T = md.use_out ? h.min_out : h.min_d;
-      if (far > 0 && T > nv.bound) {
+      if (h.far > 0 && T > nv.bound) {
+        if (threadIdx.x == 0) s_solo_cont = 0;
         // raise B: from the bucket lists when they cover T, else by a full refill
-        bool full = nv.lists == nullptr;
-        if (!full && !nf_pull(p, grp, md, k, sh, nv, &full)) return;
-        if (full) {
-          if (!nf_refill(p, grp, md, k, sh, nv, nf_uses)) return;
+        const int pulled = nv.lists == nullptr ? kNfIdle : nf_pull(k);
+        if (pulled == kNfFail) return;
+        if (pulled == kNfIdle) {
+          if (!nf_refill(k, s_nf_uses)) return;
+          if (threadIdx.x == 0) ++s_nf_uses;
           nf_code = kArmNfRefill;
         } else {
           nf_code = kArmNfPull;
         }
         h = load_head(ctl, k, nv.bound != kNoBound);
-        nF = h.nQ;
-        if (nF == 0) {  // a refill or pull always moves the vertex that attains T
-          if (leader) atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
+        if (SSSP_RARE(h.nQ == 0)) {  // a refill or pull always moves the vertex that attains T
+          if (grp.rank == 0 && threadIdx.x == 0) atomicCAS(&ctl->err, 0, (int)SSSP_ERR_INTERNAL);
           break;
         }
-      } else if (far == 0 && nv.bound == kNoBound && (uint64_t)nF >= (uint64_t)p.nf_min * grp.size &&
-                 (uint64_t)nF * 256 >= (uint64_t)p.nf_share * n) {
+      } else if (SSSP_RARE(h.far == 0 && nv.bound == kNoBound && (uint64_t)h.nQ >= (uint64_t)p.nf_min * grp.size &&
+                           (uint64_t)h.nQ * 256 >= (uint64_t)p.nf_share * p.g.n)) {
         // (with a policy too: while the fringe is split, every phase runs
         // the static sparse arm, see choose_arm)
-        if (!nf_split(p, grp, md, k, sh, nv, nf_uses)) return;
+        if (threadIdx.x == 0) s_solo_cont = 0;
+        const int split = nf_split(k, s_nf_uses);
+        if (split == kNfFail) return;
+        if (split == kNfUsed && threadIdx.x == 0) ++s_nf_uses;
         h = load_head(ctl, k, nv.bound != kNoBound);
-        nF = h.nQ;
         if (nv.bound != kNoBound) nf_code = kArmNfRefill;
       }
       if (nv.bound != kNoBound) nf_code |= kArmNfActive;
-    } else if (nF == 0) {
+    } else if (h.nQ == 0) {
       break;
     }
-    const bool fast_solo = md.fused && !dense_forced && nF <= solo_cap;
-    const bool generic_solo = !md.fused && grp.size > 1 && nF <= p.solo_max;
-    if (fast_solo || generic_solo) {
-      __shared__ unsigned long long s_next;
-      __shared__ int s_ok, s_resume;
-      bool resume_relax = false;
+    // (a phase after one that had too many edges for one block probably has so
+    // too, and an episode that only selects costs more than a grid phase; a
+    // policy's phases keep to the fringe's size)
+    const bool fast_solo = md.fused && (p.crit & SSSP_FRONTIER_DENSE) == 0 && h.nQ <= solo_enter(p) &&
+                           (h.e_prev <= p.solo_edges || grp.size == 1 || (p.crit & SSSP_POLICY_LEARNED));
+    const bool three_step_solo = kKind == kAny && !md.fused && grp.size > 1 && h.nQ <= p.solo_max;
+    if ((fast_solo || three_step_solo) && !forced) {
+      uint64_t r;  // 4 k + kSoloResume or kSoloNoFit
       if (grp.rank == 0) {
-        if (fast_solo) {
-          k = solo_episode(pk, md, k, nv, nf_code, smem, st, grp.size > 1, &resume_relax);
-        } else {
-          // three-step kind: the generic phase on this block alone
-          const Grp solo{grp.bar, grp.err, grp.limit, 0, 1};
-          while (nF != 0 && nF <= p.solo_max && k <= (uint64_t)n + 1) {
-            run_phase(p, solo, md, k, nv, 0u, h, sh, st);
-            ++k;
-            if (tid == 0) ctl->heartbeat = k;
-            h = load_head(ctl, k, nv.bound != kNoBound);
-            nF = h.nQ;
-          }
-        }
-        if (grp.size > 1) {
-          __syncthreads();
-          if (tid == 0) {
-            ctl->next_phase = k;
-            ctl->resume_relax = resume_relax ? 1u : 0u;
-            __threadfence();
-            red_release_gpu_add(&ctl->gate, 1u);
-          }
-          __syncthreads();
-        }
+        const bool group = grp.size > 1, narrow = kKind != kAny || p.g.max_w <= kSoloNarrowW, split = nv.bound != kNoBound;
+        const uint32_t k32 = (uint32_t)k;
+        if (kKind == kAny && !md.fused) r = 4 * generic_solo(k);
+        else if (narrow) r = split ? solo_episode<true, uint32_t, kKind>(k32, nf_code, group)
+                                   : solo_episode<false, uint32_t, kKind>(k32, nf_code, group);
+        else r = split ? solo_episode<true, unsigned long long, kKind>(k32, nf_code, group)
+                       : solo_episode<false, unsigned long long, kKind>(k32, nf_code, group);
+        if (group) episode_end(r);
       } else {
-        if (tid == 0) {
-          s_ok = bounded_wait_change(&ctl->gate, episodes, grp.limit, grp.err, &ctl->heartbeat) ? 1 : 0;
-          s_next = ld_relaxed_gpu_u64(&ctl->next_phase);
-          s_resume = (int)ldcg_u32(&ctl->resume_relax);
-        }
-        __syncthreads();
-        if (!s_ok) return;
-        k = s_next;
-        resume_relax = s_resume != 0;
-        __syncthreads();
+        r = episode_wait(episodes);
+        if (r == 0) return;
       }
       ++episodes;
-      if (resume_relax) {
+      k = r >> 2;
+      forced = (r & kSoloNoFit) != 0;
+      if (r & kSoloResume) {
         const Arm arm = arm_for(p, ldcg_u32(&ctl->slot[k % 4].qcount));
-        const bool ok = nv.bound != kNoBound ? phase_relax<true>(p, grp, md, arm, k, nv, true, sh, st)
-                                             : phase_relax<false>(p, grp, md, arm, k, nv, true, sh, st);
-        if (!ok) return;
+        if (!(nv.bound != kNoBound ? phase_relax<true, kKind>(false, arm, k, true)
+                                   : phase_relax<false, kKind>(false, arm, k, true)))
+          return;
         ++k;
       }
       continue;
     }
-    if (!run_phase(p, grp, md, k, nv, nf_code, h, sh, st)) return;
+    forced = false;
+    if (threadIdx.x == 0) s_solo_cont = 0;
+    if (!run_phase<kKind>(false, k, nf_code, h)) return;
     ++k;
   }
-  if (leader) {
-    ctl->phases = st.phases;
-    ctl->sum_f = st.sum_f;
-    ctl->settled = st.settled;
-    ctl->relaxed = st.relaxed;
-  }
-  if (!grp.sync()) return;
-  for (uint64_t v = gtid; v < n; v += gthreads) {
-    const unsigned long long d = ldcg_u64(&w.vrec[v].d) & ~kSettledBit;
-    w.dist[v] = d == kUnexplored ? kInf64 : d;
-  }
+  solve_finish();
 }
 
 // The solve's parameters live in shared memory, one copy per block: every
 // step reads them through a reference, and a per-thread copy in local memory
 // would take L1 space (and L2 traffic) from the graph's data.
+template <int kKind>
 __global__ void __launch_bounds__(kThreads, 1) k_solve_grid(SolveParams p) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ SolveParams s_p;
   grid_sync_init();
   if (threadIdx.x == 0) s_p = p;
   __syncthreads();
   const Grp grp{&s_p.ws.ctl->bar, &s_p.ws.ctl->err, s_p.wait_ns, blockIdx.x, gridDim.x};
-  solve_body(s_p, p, grp, smem);
+  solve_body<kKind>(grp);
 }
 
-// Batched solver: the grid is split into groups of `bpg` blocks; the first
-// block of a group takes the next solve from a device counter (descriptors
-// sorted largest first by the host) and the group runs it to the end.
+// Batched solver: the grid is split into groups of blocks; the first block of a
+// group takes the next solve from a device counter (descriptors sorted largest
+// first by the host) and the group runs it to the end.  A launch may have
+// several stages, each with a range of the solves, its own group size and its
+// own counter: a block that finds the counter of one stage run out goes on with
+// the next.
 struct BatchItem {
   GraphView g;
   SolveWS ws;
@@ -2195,57 +2567,87 @@ struct GroupSlot {
   unsigned int pad;
 };
 
+constexpr uint32_t kMaxStages = 5;
+struct BatchStages {
+  uint32_t count;
+  uint32_t bpg[kMaxStages];    // blocks per solve
+  uint32_t end[kMaxStages];    // solves [end of the last stage, end)
+  uint32_t slot[kMaxStages];   // first group slot
+};
+
 // Execution tuning of a batch launch (see sssp_tuning).
 struct BatchTuning {
   uint32_t solo_max, solo_edges, nf_min, nf_target, nf_share;
+  uint32_t solo_spt, pol_off;
 };
 
-__global__ void __launch_bounds__(kThreads) k_solve_batch(const BatchItem* items, uint32_t count,
-                                                           unsigned int* next, GroupSlot* groups, uint32_t bpg,
-                                                           uint32_t crit, BatchTuning tu,
-                                                           unsigned long long wait_ns, int* err,
-                                                           unsigned long long* phases_out, const float* policy) {
-  extern __shared__ __align__(16) unsigned char smem[];
+// kT threads per block, as many blocks per SM as its registers hold: see
+// batch_threads.
+template <int kKind, int kT>
+__global__ void __launch_bounds__(kT, kThreads / kT) k_solve_batch(const BatchItem* items, unsigned int* next, GroupSlot* groups, BatchStages stages, uint32_t crit,
+              BatchTuning tu, unsigned long long wait_ns, int* err, unsigned long long* phases_out, const float* policy) {
   __shared__ unsigned int s_item;
-  grid_sync_init();
-  const unsigned int gidx = blockIdx.x / bpg, rank = blockIdx.x % bpg;
-  GroupSlot* gs = &groups[gidx];
-  const Grp grp{&gs->bar, err, wait_ns, rank, bpg};
-  for (;;) {
-    if (rank == 0 && threadIdx.x == 0) gs->item = atomicAdd(next, 1u);
-    if (!grp.sync()) return;
-    if (threadIdx.x == 0) s_item = ldcg_u32(&gs->item);
+  for (uint32_t stage = 0; stage < stages.count; ++stage) {
+    const uint32_t bpg = stages.bpg[stage], begin = stage ? stages.end[stage - 1] : 0u, end = stages.end[stage];
+    const unsigned int gidx = blockIdx.x / bpg, rank = blockIdx.x % bpg;
+    if (gidx >= gridDim.x / bpg) continue;  // (a block left over)
+    GroupSlot* gs = &groups[stages.slot[stage] + gidx];
+    const Grp grp{&gs->bar, err, wait_ns, rank, bpg};
     __syncthreads();
-    const unsigned int it = s_item;
-    if (!grp.sync()) return;  // everyone has read the mailbox before it is reused
-    if (it >= count) break;
-    __shared__ SolveParams p;  // one copy per block (see k_solve_grid)
-    if (threadIdx.x == 0) {
-      p.g = items[it].g;
-      p.ws = items[it].ws;
-      p.source = items[it].source;
-      p.crit = crit;
-      p.wait_ns = wait_ns;
-      p.solo_max = tu.solo_max;
-      p.solo_edges = tu.solo_edges;
-      p.nf_min = tu.nf_min;
-      p.nf_target = tu.nf_target;
-      p.nf_share = tu.nf_share;
-      p.policy = policy;
-    }
-    __syncthreads();
-    solve_body(p, p, grp, smem);
-    if (*(volatile int*)err != 0) return;
-    if (rank == 0 && threadIdx.x == 0) {
-      const int e = (int)ldcg_u32(reinterpret_cast<const uint32_t*>(&p.ws.ctl->err));
-      if (e != 0) atomicCAS(err, 0, e);
-      if (phases_out) phases_out[items[it].out_index] = p.ws.ctl->phases;
+    grid_sync_init();
+    for (;;) {
+      if (rank == 0 && threadIdx.x == 0) gs->item = atomicAdd(&next[stage], 1u);
+      if (!grp.sync()) return;
+      if (threadIdx.x == 0) s_item = ldcg_u32(&gs->item);
+      __syncthreads();
+      const unsigned int it = begin + s_item;
+      if (!grp.sync()) return;  // everyone has read the mailbox before it is reused
+      if (it >= end) break;
+      if (threadIdx.x == 0) {
+        SolveParams& p = s_p;
+        p.g = items[it].g;
+        p.ws = items[it].ws;
+        p.source = items[it].source;
+        p.crit = crit;
+        p.wait_ns = wait_ns;
+        p.solo_max = tu.solo_max;
+        p.solo_edges = tu.solo_edges;
+        p.nf_min = tu.nf_min;
+        p.nf_target = tu.nf_target;
+        p.nf_share = tu.nf_share;
+        p.solo_spt = tu.solo_spt;
+        p.pol_off = tu.pol_off;
+        p.policy = policy;
+      }
+      __syncthreads();
+      solve_body<kKind>(grp);
+      if (*(volatile int*)err != 0) return;
+      if (rank == 0 && threadIdx.x == 0) {
+        const int e = (int)ldcg_u32(reinterpret_cast<const uint32_t*>(&s_p.ws.ctl->err));
+        if (e != 0) atomicCAS(err, 0, e);
+        if (phases_out) phases_out[items[it].out_index] = s_p.ws.ctl->phases;
+      }
     }
   }
 }
 
 // ---------------------------------------------------------------------------
 // host side
+
+// The kernel instance for a criterion mask (see kAny).
+int kind_of(uint32_t crit, bool narrow, bool records) {
+  constexpr uint32_t is = SSSP_IN_STATIC | SSSP_OUT_STATIC;
+  constexpr uint32_t arms = is | SSSP_IN_SIMPLE | SSSP_POLICY_LEARNED | SSSP_FRONTIER_DENSE | SSSP_FRONTIER_AUTO;
+  if (!narrow || records || (crit & ~arms)) return kAny;
+  return (crit & ~is) ? kArms : kStatic;
+}
+int solve_kind(const SolveParams& p) {
+  return kind_of(p.crit, p.g.max_w <= kSoloNarrowW, p.ws.trace || p.ws.settle_phase || !p.ws.tile_owner);
+}
+const void* grid_kernel(int kind) {
+  return kind == kStatic ? (const void*)k_solve_grid<kStatic>
+                         : kind == kArms ? (const void*)k_solve_grid<kArms> : (const void*)k_solve_grid<kAny>;
+}
 
 namespace {
 
@@ -2266,18 +2668,33 @@ int current_device() {
   return dev;
 }
 
+template <int kT>
+const void* batch_kernel_of(int kind) {
+  return kind == kStatic ? (const void*)k_solve_batch<kStatic, kT>
+                         : kind == kArms ? (const void*)k_solve_batch<kArms, kT> : (const void*)k_solve_batch<kAny, kT>;
+}
+const void* batch_kernel(int kind, uint32_t threads) {
+  return threads == kThreads ? batch_kernel_of<kThreads>(kind) : batch_kernel_of<kSmallThreads>(kind);
+}
+
 sssp_status ensure_kernel_attrs() {
   const int dev = current_device();
   if (dev < 0 || dev >= kMaxDevices) return fail(SSSP_ERR_CUDA, "no usable current CUDA device (ordinal %d)", dev);
   if (g_blocks_per_sm[dev].load() > 0) return SSSP_OK;
   std::lock_guard<std::mutex> lock(g_attr_mu);
   if (g_blocks_per_sm[dev].load() > 0) return SSSP_OK;
-  SSSP_CUDA_TRY(cudaFuncSetAttribute(k_solve_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
-  SSSP_CUDA_TRY(cudaFuncSetAttribute(k_solve_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
-  int a = 0, b = 0;
-  SSSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_solve_grid, kThreads, kSmemBytes));
-  SSSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_solve_batch, kThreads, kSmemBytes));
-  const int per_sm = std::min(a, b);
+  int per_sm = 1 << 10;
+  for (int kind : {kAny, kArms, kStatic}) {
+    for (const void* kernel : {grid_kernel(kind), batch_kernel(kind, kThreads), batch_kernel(kind, kSmallThreads)}) {
+      const bool small = kernel == batch_kernel(kind, kSmallThreads);
+      const int threads = small ? kSmallThreads : kThreads;
+      const size_t smem = small ? kMaxSmallSmem : kMaxSmem;
+      SSSP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      int a = 0;
+      SSSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, kernel, threads, smem));
+      per_sm = std::min(per_sm, small ? a / (kThreads / kSmallThreads) : a);
+    }
+  }
   if (per_sm < 1) return fail(SSSP_ERR_CUDA, "solve kernel cannot be resident");
   g_blocks_per_sm[dev].store(per_sm);
   return SSSP_OK;
@@ -2318,6 +2735,39 @@ int blocks_for(uint32_t n) {
 }
 
 }  // namespace
+
+namespace {
+
+// Shared-memory layout of a launch (P: SolveParams or BatchTuning); returns its
+// dynamic shared memory (at most kMaxSmem).  `large`: solo_large of all its
+// graphs; `narrow`: no edge of them costs more than kSoloNarrowW.
+template <class P>
+size_t solo_shape_of(bool large, bool narrow, uint32_t crit, uint32_t threads, P* p) {
+  const bool policy = (crit & SSSP_POLICY_LEARNED) != 0, small_block = threads != kThreads;
+  p->solo_spt = small_block ? (!large ? kSmallSpt : narrow ? kSmallLargeSpt : kSmallLargeWideSpt)
+                            : (!large ? kSoloSmallSpt : narrow ? kSoloLargeSpt : kSoloLargeWideSpt);
+  const size_t solo = (size_t)threads * (p->solo_spt * (narrow ? kSoloSlotBytes : kSoloWideSlotBytes) +
+                                         sizeof(uint32_t)) + threads / 32 * kSoloList * sizeof(uint4);
+  p->pol_off = (uint32_t)((std::max(kGridSmem, solo) + 15) / 16 * 16);
+  return p->pol_off + (policy ? kPolicySmem : 0);
+}
+
+// Graphs of at most kSoloLargeN vertices, or with fewer than 6 edges a vertex
+// (meshes and the like, whose fringes stay small for many phases), get twice the
+// slots: their solves live in episodes.  On larger and denser ones the grid
+// phases count, and these want the L1 that the slots would take.  (G(2^14, 2^17)
+// with 4, 8, 12, 16 slots a thread: 1.47, 1.37, 1.43, 1.64 ms; the 1024 x 1024
+// grid 110.7, 108.9, 110.4, 110.3.)  In blocks of kSmallThreads, two to an SM,
+// the meshes alone: 200 solves of G(20000, 160000) take 5.5 ms with 16 slots a
+// thread, 4.2 with 8, and 256 sources on the 512 x 512 grid 48 and 73.
+bool solo_mesh(uint32_t n, uint64_t m) { return m < 6ull * n; }
+bool solo_large(uint32_t n, uint64_t m) { return n <= kSoloLargeN || solo_mesh(n, m); }
+
+}  // namespace
+
+size_t solo_shape(uint32_t crit, SolveParams* p) {
+  return solo_shape_of(solo_large(p->g.n, p->g.m), p->g.max_w <= kSoloNarrowW, crit, kThreads, p);
+}
 
 void workspace_free(Workspace* ws) {
   if (!ws) return;
@@ -2450,11 +2900,12 @@ sssp_status solve_one(sssp_graph* g, uint32_t source, uint32_t crit, uint64_t* d
   p.nf_share = nearfar_share();
   p.policy = (crit & SSSP_POLICY_LEARNED) ? policy_weights() : nullptr;
 
+  const size_t smem = solo_shape(crit, &p);
   const int blocks = blocks_for(g->n);
   SSSP_CUDA_TRY(cudaMemsetAsync(ws->ctl, 0, sizeof(Ctl), st));
   void* args[] = {&p};
-  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve_grid, dim3(blocks), dim3(kThreads), args,
-                                            kSmemBytes, st));
+  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel(grid_kernel(solve_kind(p)), dim3(blocks), dim3(kThreads), args,
+                                            smem, st));
   SSSP_CUDA_TRY(cudaMemcpyAsync(ws->ctl_host, ws->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   if (!dist_dev)
     SSSP_CUDA_TRY(cudaMemcpyAsync(dist_out, ws->dist, g->n * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
@@ -2484,9 +2935,13 @@ sssp_status solve_one(sssp_graph* g, uint32_t source, uint32_t crit, uint64_t* d
 struct BatchPlan {
   uint32_t count = 0;
   uint32_t crit = 0;
+  bool large = true, mesh = true, narrow = true;  // see solo_shape_of
+  uint32_t recording = 0;              // solves with a trace or settle phases attached
+  int kind() const { return kind_of(crit, narrow, recording != 0); }
   uint32_t bpg = 1;                    // blocks per solve
-  uint32_t groups = 0;
-  uint32_t max_groups = 0;             // gslots allocated (any bpg >= 1 fits)
+  bool staged = false;                 // bpg = 1: larger solves get more blocks
+  uint32_t slots = 0;                  // gslots allocated (any stages fit)
+  std::vector<uint64_t> size;          // m + n of the solves, largest first
   BatchItem* items = nullptr;          // device, largest graph first
   unsigned int* next = nullptr;        // device work counter
   GroupSlot* gslots = nullptr;         // device, one per group
@@ -2521,26 +2976,95 @@ void batch_free(sssp_batch* b) {
   delete b;
 }
 
+// Launch plan of a batch: threads per block, blocks and stages.
+//
+// One block per solve is the most efficient use of the GPU (two are 1.4 to 1.8
+// times as fast, eight 2 to 4.5 times), but a launch then takes at least as long
+// as its largest solve.  Solves larger than an SM's share of the batch's edges
+// get 2, 4, 8 or 16 blocks, in stages before the rest: 256 uneven graphs (2^10
+// to 2^18 vertices) with one source each 37.6 -> 24.6 ms, with four each, where
+// only the largest few are above the share, 53 -> 51.7 ms.  With a half or a
+// quarter of the share as the limit, four sources take 54 and 60 ms.  Meshes
+// keep to one block, which runs their small fringes fastest, and a policy's
+// batches to one size, on which its choices depend.
+//
+// More solves than SMs and of about one size (the largest at most twice the
+// mean) run in blocks of kSmallThreads, two to an SM, whose latency chains
+// overlap: 256 sources on the 512 x 512 grid 72 -> 48 ms, 200 solves of G(20000,
+// 160000) 5.0 -> 4.2 ms, of G(100000, 800000) 21.8 -> 19.5, 256 of G(1500,
+// 12000) 0.71 -> 0.59.  Of uneven sizes, the largest ones would take twice as
+// long (the 256 graphs with four sources 59 ms at best).
+struct LaunchPlan {
+  uint32_t threads, blocks;
+  BatchStages stages;
+};
+LaunchPlan batch_plan(const BatchPlan& b) {
+  const uint32_t resident = resident_blocks();
+  LaunchPlan l;
+  memset(&l, 0, sizeof l);
+  l.threads = kThreads;
+  auto stage = [&](uint32_t bpg, uint32_t end) {
+    const uint32_t i = l.stages.count, begin = i ? l.stages.end[i - 1] : 0u;
+    if (end <= begin) return;
+    l.stages.bpg[i] = bpg;
+    l.stages.end[i] = end;
+    l.stages.slot[i] = i ? l.stages.slot[i - 1] + l.blocks / l.stages.bpg[i - 1] : 0u;
+    ++l.stages.count;
+  };
+  if (!b.staged) {
+    l.blocks = std::max<uint32_t>(1, std::min<uint32_t>(b.count, resident / b.bpg)) * b.bpg;
+    stage(b.bpg, b.count);
+    return l;
+  }
+  uint64_t total = 0;
+  for (uint64_t x : b.size) total += x;
+  if (b.count > resident && b.size[0] * b.count <= 2 * total) l.threads = kSmallThreads;
+  l.blocks = std::min<uint32_t>(b.count, resident * (kThreads / l.threads));
+  if (l.threads == kThreads && !b.mesh && !(b.crit & SSSP_POLICY_LEARNED)) {
+    const uint64_t share = std::max<uint64_t>(1, total / l.blocks);
+    for (uint32_t bpg = 16; bpg > 1; bpg /= 2) {
+      uint32_t end = l.stages.count ? l.stages.end[l.stages.count - 1] : 0u;
+      while (end < b.count && bpg <= resident && b.size[end] > share * (bpg / 2) &&
+             b.h_items[end].g.n > kVertsPerBlock * (bpg / 2))
+        ++end;
+      if (end > 0) l.blocks = resident;
+      stage(bpg, end);
+    }
+  }
+  stage(1, b.count);
+  return l;
+}
+
 // Queue the batch on `st`: reset the work counter, group slots and every
 // control block, then one cooperative launch whose groups pull solves.
 sssp_status batch_enqueue(sssp_batch* b, cudaStream_t st) {
-  SSSP_CUDA_TRY(cudaMemsetAsync(b->next, 0, sizeof(unsigned int), st));
-  SSSP_CUDA_TRY(cudaMemsetAsync(b->gslots, 0, b->groups * sizeof(GroupSlot), st));
+  LaunchPlan l = batch_plan(*b);
+  SSSP_CUDA_TRY(cudaMemsetAsync(b->next, 0, kMaxStages * sizeof(unsigned int), st));
+  SSSP_CUDA_TRY(cudaMemsetAsync(b->gslots, 0, b->slots * sizeof(GroupSlot), st));
   SSSP_CUDA_TRY(cudaMemsetAsync(b->err, 0, sizeof(int), st));
   for (Workspace* w : b->ws) SSSP_CUDA_TRY(cudaMemsetAsync(w->ctl, 0, sizeof(Ctl), st));
-  const int blocks = (int)(b->groups * b->bpg);
-  BatchTuning tu{solo_max(), solo_edges(), nearfar_min(), nearfar_target(), nearfar_share()};
+  BatchTuning tu{solo_max(), solo_edges(), nearfar_min(), nearfar_target(), nearfar_share(), 0, 0};
+  const size_t smem = solo_shape_of(l.threads == kThreads ? b->large : b->mesh, b->narrow, b->crit, l.threads, &tu);
   unsigned long long wait = wait_limit_ns();
-  void* args[] = {&b->items, &b->count, &b->next, &b->gslots, &b->bpg, &b->crit, &tu, &wait, &b->err, &b->phases,
-                  &b->policy};
-  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve_batch, dim3(blocks), dim3(kThreads), args,
-                                            kSmemBytes, st));
+  void* args[] = {&b->items, &b->next, &b->gslots, &l.stages, &b->crit, &tu, &wait, &b->err, &b->phases, &b->policy};
+  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel(batch_kernel(b->kind(), l.threads), dim3(l.blocks), dim3(l.threads), args,
+                                            smem, st));
   return SSSP_OK;
 }
 
+// Blocks per solve for a batch: as many groups as solves while that keeps
+// every resident block busy, fewer (larger) groups for few large solves.
+uint32_t choose_bpg(sssp_graph* const* graphs, uint32_t count) {
+  const uint32_t resident = resident_blocks();
+  uint64_t maxn = 0;
+  for (uint32_t i = 0; i < count; ++i) maxn = std::max<uint64_t>(maxn, graphs[i]->n);
+  const uint32_t bpg = std::max<uint32_t>(1, resident / std::max<uint32_t>(1, count));
+  const uint32_t useful = (uint32_t)std::max<uint64_t>(1, (maxn + kVertsPerBlock - 1) / kVertsPerBlock);
+  return std::min(bpg, useful);
+}
+
 sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint32_t count, uint32_t crit,
-                        uint64_t* const* dist_out, uint64_t* phases_dev, uint32_t bpg, cudaStream_t st,
-                        sssp_batch** out) {
+                        uint64_t* const* dist_out, uint64_t* phases_dev, cudaStream_t st, sssp_batch** out) {
   if (!graphs || !sources || !dist_out || count == 0) return fail(SSSP_ERR_INVALID_ARG, "empty or NULL batch");
   for (uint32_t i = 0; i < count; ++i) {
     if (!graphs[i]) return fail(SSSP_ERR_INVALID_ARG, "graph %u is NULL", i);
@@ -2553,15 +3077,20 @@ sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint
   sssp_status s = ensure_kernel_attrs();
   if (s != SSSP_OK) return s;
   const uint32_t resident = resident_blocks();
-  if (bpg == 0) bpg = 1;
-  if (bpg > resident) bpg = resident;
+  const uint32_t tuned = batch_blocks_per_solve();
+  const uint32_t bpg = std::min(tuned ? tuned : choose_bpg(graphs, count), resident);
   sssp_batch* b = new (std::nothrow) sssp_batch();
   if (!b) return fail(SSSP_ERR_OUT_OF_MEMORY, "host allocation failed");
   b->count = count;
   b->crit = crit;
+  for (uint32_t i = 0; i < count; ++i) {
+    b->large = b->large && solo_large(graphs[i]->n, graphs[i]->m);
+    b->mesh = b->mesh && solo_mesh(graphs[i]->n, graphs[i]->m);
+    b->narrow = b->narrow && graphs[i]->max_w <= kSoloNarrowW;
+  }
   b->bpg = bpg;
-  b->groups = std::max<uint32_t>(1, std::min<uint32_t>(count, resident / bpg));
-  b->max_groups = std::max<uint32_t>(1, std::min(count, resident));
+  b->staged = !tuned && bpg == 1;
+  b->slots = kMaxStages * resident * (kThreads / kSmallThreads);
   // Largest solves first, so the tail of the queue holds the short ones.
   std::vector<uint32_t> order(count);
   for (uint32_t i = 0; i < count; ++i) order[i] = i;
@@ -2581,9 +3110,10 @@ sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint
     h[k].ws = ws_view(b->ws[k], reinterpret_cast<unsigned long long*>(dist_out[i]), crit, graphs[i]->rrow_off);
     h[k].source = sources[i];
     h[k].out_index = i;
+    b->size.push_back(graphs[i]->m + graphs[i]->n);
   }
-  if ((s = dev_alloc(&b->items, count)) != SSSP_OK || (s = dev_alloc(&b->next, 1)) != SSSP_OK ||
-      (s = dev_alloc(&b->gslots, std::max<uint32_t>(1, std::min(count, resident)))) != SSSP_OK ||
+  if ((s = dev_alloc(&b->items, count)) != SSSP_OK || (s = dev_alloc(&b->next, kMaxStages)) != SSSP_OK ||
+      (s = dev_alloc(&b->gslots, b->slots)) != SSSP_OK ||
       (s = dev_alloc(&b->err, 1)) != SSSP_OK) {
     batch_free(b);
     return s;
@@ -2636,22 +3166,20 @@ sssp_status batch_capture(sssp_batch* b) {
   return SSSP_OK;
 }
 
+// Capture it anew (no launch of the batch is in flight).
+sssp_status batch_recapture(sssp_batch* b) {
+  if (b->exec) cudaGraphExecDestroy(b->exec);
+  if (b->graph) cudaGraphDestroy(b->graph);
+  b->exec = nullptr;
+  b->graph = nullptr;
+  return batch_capture(b);
+}
+
 sssp_status batch_status(sssp_batch* b) {
   int e = 0;
   SSSP_CUDA_TRY(cudaMemcpy(&e, b->err, sizeof(int), cudaMemcpyDeviceToHost));
   if (e != 0) return fail((sssp_status)e, "device-side error %d in a batched solve", e);
   return SSSP_OK;
-}
-
-// Blocks per solve for a batch: as many groups as solves while that keeps
-// every resident block busy, fewer (larger) groups for few large solves.
-uint32_t choose_bpg(sssp_graph* const* graphs, uint32_t count) {
-  const uint32_t resident = resident_blocks();
-  uint64_t maxn = 0;
-  for (uint32_t i = 0; i < count; ++i) maxn = std::max<uint64_t>(maxn, graphs[i]->n);
-  const uint32_t bpg = std::max<uint32_t>(1, resident / std::max<uint32_t>(1, count));
-  const uint32_t useful = (uint32_t)std::max<uint64_t>(1, (maxn + kVertsPerBlock - 1) / kVertsPerBlock);
-  return std::min(bpg, useful);
 }
 
 }  // namespace
@@ -2684,8 +3212,7 @@ extern "C" sssp_status sssp_solve_batch(sssp_graph* const* graphs, const uint32_
   for (uint32_t i = 0; i < count; ++i)
     if (!graphs[i]) return fail(SSSP_ERR_INVALID_ARG, "graph %u is NULL", i);
   sssp_batch* b = nullptr;
-  const uint32_t bpg = batch_blocks_per_solve() ? batch_blocks_per_solve() : choose_bpg(graphs, count);
-  s = batch_build(graphs, sources, count, criterion, dist_out, ph_dev ? phases_out : nullptr, bpg, st, &b);
+  s = batch_build(graphs, sources, count, criterion, dist_out, ph_dev ? phases_out : nullptr, st, &b);
   if (s != SSSP_OK) return s;
   s = batch_enqueue(b, st);
   if (s == SSSP_OK && cudaStreamSynchronize(st) != cudaSuccess) s = fail(SSSP_ERR_CUDA, "batched solve failed");
@@ -2711,8 +3238,7 @@ extern "C" sssp_status sssp_batch_create(sssp_graph* const* graphs, const uint32
     if (!graphs[i]) return fail(SSSP_ERR_INVALID_ARG, "graph %u is NULL", i);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   sssp_batch* b = nullptr;
-  const uint32_t bpg = batch_blocks_per_solve() ? batch_blocks_per_solve() : choose_bpg(graphs, count);
-  s = batch_build(graphs, sources, count, criterion, dist_out, phases_out, bpg, st, &b);
+  s = batch_build(graphs, sources, count, criterion, dist_out, phases_out, st, &b);
   if (s != SSSP_OK) return s;
   if ((s = batch_capture(b)) != SSSP_OK) {
     batch_free(b);
@@ -2738,6 +3264,7 @@ extern "C" sssp_status sssp_batch_autotune(sssp_batch* b, void* stream, uint32_t
   constexpr int kTimed = 3;
   constexpr float kWarmCut = 1.5f, kStopCut = 1.1f, kKeepOwn = 0.97f;
   const uint32_t bpg0 = b->bpg;
+  const bool own = b->staged;  // (the batch's own choice is a staged one)
   std::vector<uint32_t> ladder;
   for (uint32_t c = 1; c < resident; c *= 2) ladder.push_back(c);
   ladder.push_back(resident);
@@ -2753,7 +3280,7 @@ extern "C" sssp_status sssp_batch_autotune(sssp_batch* b, void* stream, uint32_t
   // the warm-up alone was kWarmCut times the best median
   auto measure = [&](uint32_t c, float* out) -> sssp_status {
     b->bpg = c;
-    b->groups = std::max<uint32_t>(1, std::min<uint32_t>(b->count, resident / c));
+    b->staged = own && c == bpg0;
     sssp_status r = SSSP_OK;
     if (cudaEventRecord(ev[0], st) != cudaSuccess) return fail(SSSP_ERR_CUDA, "timing a batch launch failed");
     if ((r = batch_enqueue(b, st)) != SSSP_OK) return r;  // warm-up
@@ -2795,12 +3322,8 @@ extern "C" sssp_status sssp_batch_autotune(sssp_batch* b, void* stream, uint32_t
   }
   for (auto& e : ev) cudaEventDestroy(e);
   b->bpg = s == SSSP_OK ? best : bpg0;
-  b->groups = std::max<uint32_t>(1, std::min<uint32_t>(b->count, resident / b->bpg));
-  if (b->exec) cudaGraphExecDestroy(b->exec);
-  if (b->graph) cudaGraphDestroy(b->graph);
-  b->exec = nullptr;
-  b->graph = nullptr;
-  const sssp_status sc = batch_capture(b);
+  b->staged = own && b->bpg == bpg0;
+  const sssp_status sc = batch_recapture(b);
   if (s != SSSP_OK) return s;
   if (sc != SSSP_OK) return sc;
   if (bpg_out) *bpg_out = best;
@@ -2819,13 +3342,16 @@ extern "C" sssp_status sssp_batch_trace(sssp_batch* b, uint32_t i, sssp_phase_re
   while (k < b->count && b->h_items[k].out_index != i) ++k;
   if (k == b->count) return fail(SSSP_ERR_INTERNAL, "solve %u has no descriptor", i);
   BatchItem& it = b->h_items[k];
+  const bool was = it.ws.trace || it.ws.settle_phase;
+  const int kind = b->kind();
   it.ws.trace = trace_cap ? trace : nullptr;
   it.ws.trace_cap = trace ? trace_cap : 0;
   it.ws.settle_phase = settle_phase;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  b->recording += (it.ws.trace || it.ws.settle_phase ? 1u : 0u) - (was ? 1u : 0u);
   SSSP_CUDA_TRY(cudaMemcpyAsync(&b->items[k], &it, sizeof(BatchItem), cudaMemcpyHostToDevice, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));
-  return SSSP_OK;
+  return b->kind() == kind ? SSSP_OK : batch_recapture(b);  // (the other kernel from now on)
 }
 
 extern "C" sssp_status sssp_batch_launch(sssp_batch* b, void* stream) {

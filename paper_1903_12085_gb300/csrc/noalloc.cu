@@ -59,9 +59,9 @@ sssp_status setup_for_current_device(DeviceSetup** out) {
   if (!s.ready) {
     void* p = nullptr;
     SSSP_CUDA_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch));
-    SSSP_CUDA_TRY(cudaFuncSetAttribute(k_solve_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
-    int per_sm = 0;
-    SSSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_grid, kThreads, kSmemBytes));
+    int per_sm = 0;  // (no tile marks: the instance that serves everything)
+    SSSP_CUDA_TRY(cudaFuncSetAttribute(grid_kernel(0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+    SSSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grid_kernel(0), kThreads, kMaxSmem));
     if (per_sm < 1) return fail(SSSP_ERR_CUDA, "solve kernel cannot be resident");
     s.base = static_cast<unsigned char*>(p);
     s.max_blocks = per_sm * sm_count();
@@ -82,7 +82,8 @@ __global__ void k_noalloc_minima_init(uint32_t n, uint32_t* out_min, uint32_t* i
 // (bad[0] set on an out-of-range target, a reserved cost or bad offsets).
 __global__ void k_noalloc_minima(uint32_t n, uint64_t m, const uint64_t* __restrict__ ro,
                                  const uint2* __restrict__ edges, uint32_t* out_min, uint32_t* in_min,
-                                 uint2* rowdeg, int* bad) {
+                                 uint2* rowdeg, int* bad, unsigned int* max_w) {
+  uint32_t top = 0;
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -100,6 +101,7 @@ __global__ void k_noalloc_minima(uint32_t n, uint64_t m, const uint64_t* __restr
         continue;
       }
       best = ed.y < best ? ed.y : best;
+      top = max(top, ed.y);
       red_min_u32(&in_min[ed.x], ed.y);
     }
     best = __reduce_min_sync(0xFFFFFFFFu, best);
@@ -108,6 +110,8 @@ __global__ void k_noalloc_minima(uint32_t n, uint64_t m, const uint64_t* __restr
       rowdeg[u] = make_uint2((uint32_t)b, (uint32_t)(e - b));
     }
   }
+  top = __reduce_max_sync(0xFFFFFFFFu, top);
+  if (lane == 0 && top > 0) atomicMax(max_w, top);
 }
 
 }  // namespace
@@ -152,10 +156,13 @@ extern "C" sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t
   SSSP_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
   const int blocks = dev->max_blocks;
   k_noalloc_minima_init<<<blocks, 256, 0, st>>>(n, out_min, in_min);
-  k_noalloc_minima<<<blocks, 256, 0, st>>>(n, m, row_offsets, e2, out_min, in_min, rowdeg, &ctl->err);
+  k_noalloc_minima<<<blocks, 256, 0, st>>>(n, m, row_offsets, e2, out_min, in_min, rowdeg, &ctl->err,
+                                          &ctl->nf_tmp);  // (a free word of the block)
   SSSP_CUDA_TRY(cudaGetLastError());
   int bad = 0;
+  uint32_t max_w = 0;
   SSSP_CUDA_TRY(cudaMemcpyAsync(&bad, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SSSP_CUDA_TRY(cudaMemcpyAsync(&max_w, &ctl->nf_tmp, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));
   if (bad) return fail(SSSP_ERR_INVALID_ARG, "sssp_solve_noalloc: invalid CSR (offsets, targets or costs)");
   SSSP_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
@@ -169,6 +176,7 @@ extern "C" sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t
   p.g.out_min = out_min;
   p.g.in_min = in_min;
   p.g.rowdeg = rowdeg;
+  p.g.max_w = max_w;
   p.ws.dist = reinterpret_cast<unsigned long long*>(dist_out);
   p.ws.vrec = reinterpret_cast<VRec*>(base + kOffVrec);
   p.ws.status = base + kOffStatus;
@@ -187,9 +195,9 @@ extern "C" sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t
   p.policy = nullptr;
   const uint64_t want = ((uint64_t)n + kVertsPerBlock - 1) / kVertsPerBlock;
   const int grid = (int)(want < (uint64_t)blocks ? (want > 0 ? want : 1) : blocks);
+  const size_t smem = solo_shape(criterion, &p);
   void* args[] = {&p};
-  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_solve_grid, dim3(grid), dim3(kThreads), args, kSmemBytes,
-                                            st));
+  SSSP_CUDA_TRY(cudaLaunchCooperativeKernel(grid_kernel(solve_kind(p)), dim3(grid), dim3(kThreads), args, smem, st));
   Ctl h;
   SSSP_CUDA_TRY(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));

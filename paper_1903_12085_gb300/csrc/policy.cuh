@@ -55,27 +55,71 @@ __host__ __device__ __forceinline__ void policy_features(float* f, uint64_t nF, 
   f[7] = (float)s_prev / (1.0f + (float)f_prev);
 }
 
-// Forward pass by one full warp: lane j owns hidden unit j of both layers.
-// Returns the 4 outputs in lanes 0..3 (broadcast to every lane via out[]).
-// `w` may point to global or shared memory (plain loads only).
-__device__ __forceinline__ void policy_forward_warp(const float* __restrict__ w, const float* f, float* out) {
-  const int lane = threadIdx.x & 31;
-  float h1 = w[kPolOffB1 + lane];
+// The same features by one full warp, feature i in lane i (i < 8; other lanes: 0):
+// one logarithm and one division in a row instead of five and eight, with the
+// same results (a scale by a power of two is exact, before or after).
+__device__ __forceinline__ float policy_feature_lane(uint32_t nF, uint32_t n, uint32_t m, uint32_t k,
+                                                     uint32_t e_prev, uint32_t s_prev, uint32_t f_prev) {
+  const int i = threadIdx.x & 31;
+  const float x = (float)(i == 0 || i == 1 ? nF : i == 2 ? e_prev : i == 4 ? k : i == 5 ? n : i == 6 ? m : s_prev);
+  const float num = i < 6 && i != 1 ? log2f(i == 5 ? x : 1.0f + x) : x;
+  const float den = i == 1 || i == 6 ? (float)n : i == 7 ? 1.0f + (float)f_prev : i == 4 || i == 5 ? 1.0f : 24.0f;
+  const float scale = i == 4 ? 1.0f / 16.0f : i == 5 || i == 6 ? 1.0f / 32.0f : 1.0f;
+  return i < kPolFeat ? num / den * scale : 0.0f;
+}
+
+// Place of weight i in a block's shared-memory copy: the matrices of the hidden
+// layers four rows at a time, so that a lane reads its column as float4s (a
+// forward pass runs with cold instruction caches, and costs what its length does).
+__device__ __forceinline__ int policy_place(int i) {
+  const int base = i < kPolOffB1 ? kPolOffW1 : kPolOffW2;
+  if ((i >= kPolOffB1 && i < kPolOffW2) || i >= kPolOffB2) return i;
+  const int r = (i - base) / kPolHidden, c = (i - base) % kPolHidden;
+  return base + (r / 4 * kPolHidden + c) * 4 + r % 4;
+}
+
+// sum += in[0..4K) * (the lane's column of a matrix placed as above), in order.
+template <int K>
+__device__ __forceinline__ float policy_column(const float* in, const float* w, float sum) {
+  const float4* const x4 = reinterpret_cast<const float4*>(in);
+  const float4* const w4 = reinterpret_cast<const float4*>(w) + (threadIdx.x & 31);
 #pragma unroll
-  for (int i = 0; i < kPolFeat; ++i) h1 = fmaf(f[i], w[kPolOffW1 + i * kPolHidden + lane], h1);
-  h1 = fmaxf(h1, 0.0f);
-  float h2 = w[kPolOffB2 + lane];
-#pragma unroll
-  for (int i = 0; i < kPolHidden; ++i)
-    h2 = fmaf(__shfl_sync(0xFFFFFFFFu, h1, i), w[kPolOffW2 + i * kPolHidden + lane], h2);
-  h2 = fmaxf(h2, 0.0f);
-#pragma unroll
-  for (int a = 0; a < kPolArms; ++a) {
-    float y = h2 * w[kPolOffW3 + lane * kPolArms + a];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xFFFFFFFFu, y, o);
-    out[a] = y + w[kPolOffB3 + a];
+  for (int q = 0; q < K; ++q) {
+    const float4 x = x4[q], c = w4[q * kPolHidden];
+    sum = fmaf(x.x, c.x, sum);
+    sum = fmaf(x.y, c.y, sum);
+    sum = fmaf(x.z, c.z, sum);
+    sum = fmaf(x.w, c.w, sum);
   }
+  return sum;
+}
+
+// Forward pass by one full warp: lane j owns hidden unit j of both layers, and
+// lane i < 8 holds feature i in `f`.  Returns the 4 outputs in out[], in every
+// lane.  `w`: the weights in shared memory (policy_place); `act`: 64 floats of
+// shared memory, 16-byte aligned like w.
+__device__ __forceinline__ void policy_forward_warp(const float* w, float f, float* act, float* out) {
+  const int lane = threadIdx.x & 31;
+  act[lane] = f;
+  __syncwarp();
+  const float h1 = policy_column<kPolFeat / 4>(act, w + kPolOffW1, w[kPolOffB1 + lane]);
+  act[kPolHidden + lane] = fmaxf(h1, 0.0f);
+  __syncwarp();
+  float h2 = policy_column<kPolHidden / 4>(act + kPolHidden, w + kPolOffW2, w[kPolOffB2 + lane]);
+  h2 = fmaxf(h2, 0.0f);
+  // the four sums over the lanes, each lane keeping the half it will own:
+  // output 2 (lane / 16) + (lane / 8) % 2
+  const float4 w3 = reinterpret_cast<const float4*>(w + kPolOffW3)[lane];
+  const float y0 = h2 * w3.x, y1 = h2 * w3.y, y2 = h2 * w3.z, y3 = h2 * w3.w;
+  const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
+  const float r0 = (hi ? y2 : y0) + __shfl_xor_sync(0xFFFFFFFFu, hi ? y0 : y2, 16);
+  const float r1 = (hi ? y3 : y1) + __shfl_xor_sync(0xFFFFFFFFu, hi ? y1 : y3, 16);
+  float r = (odd ? r1 : r0) + __shfl_xor_sync(0xFFFFFFFFu, odd ? r0 : r1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
+  r += w[kPolOffB3 + (lane >> 3)];
+#pragma unroll
+  for (int a = 0; a < kPolArms; ++a) out[a] = __shfl_sync(0xFFFFFFFFu, r, a * 8);
 }
 
 // Arm with the smallest prediction among the allowed ones (lowest index on
@@ -89,14 +133,19 @@ constexpr float kPolicyMargin = 0.35f;
 // all n vertices then costs far more per settled vertex than on the small
 // training graphs the network has seen.
 __device__ __forceinline__ int policy_pick(const float* y, bool allow_simple, bool allow_dense) {
-  const int na = allow_simple ? 4 : 2;
   int best = 0;
-  for (int a = 0; a < na; ++a) {
-    if (!isfinite(y[a])) return 0;
-    if ((a & 1) && !allow_dense) continue;
-    if (y[a] < y[best]) best = a;
+  float yb = y[0];
+  bool finite = true;
+#pragma unroll
+  for (int a = 0; a < kPolArms; ++a) {  // (unrolled, so that y stays in registers)
+    const bool may = a < 2 || allow_simple;
+    finite = finite && (!may || isfinite(y[a]));
+    if (may && (allow_dense || !(a & 1)) && y[a] < yb) {
+      best = a;
+      yb = y[a];
+    }
   }
-  return y[best] < y[0] - kPolicyMargin ? best : 0;
+  return finite && yb < y[0] - kPolicyMargin ? best : 0;
 }
 
 }  // namespace sssp
