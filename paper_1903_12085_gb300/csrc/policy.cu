@@ -7,12 +7,13 @@
 // vertex), loss = (1/B) sum_b (y_b[a_b] - t_b)^2 where y_b is the network output.
 //
 // Backward pass in two kernels:
-//   k_mlp_samples      one thread per sample: forward, then the per-sample
-//                      pre-activation gradients dZ1, dZ2, dY and the hidden
-//                      activations H1, H2 (written to scratch);
-//   k_mlp_grad_reduce  one block per weight row: dW[i][j] = sum_b A[b][i] G[b][j]
-//                      (A = X, H1 or H2; G = dZ1, dZ2 or dY), bias rows sum G;
-//                      fixed summation order, so gradients are deterministic.
+//   k_mlp_grad         a warp takes samples, two at a time, lane j as hidden
+//                      unit j of both layers, with its weights and its share of
+//                      the gradient in registers; each block adds its warps'
+//                      gradients up and writes one partial gradient;
+//   k_mlp_grad_reduce  sums the blocks' partial gradients.
+// Both in a fixed order for a given batch size and GPU, so gradients are
+// deterministic.
 #include <mutex>
 
 #include "internal.h"
@@ -50,87 +51,167 @@ __global__ void k_mlp_forward(const float* __restrict__ w, const float* __restri
   }
 }
 
-// Per-sample part of the backward pass.  Scratch layout per sample b:
-// h1[32] dz1[32] h2[32] dz2[32] dy[4] se[1].
-constexpr int kScr = 4 * kPolHidden + kPolArms + 1;
+// Gradient row of a block: the kPolWeights weight gradients, then the loss.
+constexpr int kGradRow = kPolWeights + 1;
+constexpr int kGradWarps = 8;
+constexpr int kGradTile = 8;  // samples a warp takes at a time
 
-__global__ void k_mlp_samples(const float* __restrict__ w, const float* __restrict__ x,
-                              const float* __restrict__ target, const uint32_t* __restrict__ arm, uint32_t batch,
-                              float* __restrict__ scr) {
-  __shared__ float sw[kPolWeights];
-  for (int i = threadIdx.x; i < kPolWeights; i += blockDim.x) sw[i] = w[i];
-  __syncthreads();
+// Gradient of the batch, one partial gradient per block.  Bound by the FP32
+// pipes and the latency of a sample's chain (about 115 multiply-adds a lane and
+// 24 broadcast loads of shared memory): 60,000 samples are 0.44 GFLOP, 6 us of
+// the GPU's multiply-adds, and nothing of a sample leaves the SM.  (One thread
+// a sample with its activations in local memory and 532 bytes of scratch per
+// sample, reduced by 76 blocks striding over them, took 500 us on 60,000 samples: a
+// training step 577 us, with this 55.)
+__global__ void __launch_bounds__(32 * kGradWarps, 1)
+k_mlp_grad(const float* __restrict__ w, const float* __restrict__ x, const float* __restrict__ target,
+           const uint32_t* __restrict__ arm, uint32_t batch, float* __restrict__ partial) {
+  __shared__ __align__(16) float s_x[kGradWarps][kGradTile][kPolFeat];
+  __shared__ __align__(16) float s_h[kGradWarps][2][kPolHidden], s_g[kGradWarps][2][kPolHidden];
+  __shared__ float s_grad[kGradWarps / 2][kGradRow];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float inv_b = 1.0f / (float)batch;
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x) {
-    float z1[kPolHidden], h1[kPolHidden], z2[kPolHidden], h2[kPolHidden];
-    for (int j = 0; j < kPolHidden; ++j) {
-      float z = sw[kPolOffB1 + j];
-      for (int i = 0; i < kPolFeat; ++i) z = fmaf(x[(size_t)b * kPolFeat + i], sw[kPolOffW1 + i * kPolHidden + j], z);
-      z1[j] = z;
-      h1[j] = fmaxf(z, 0.0f);
+  float w1[kPolFeat], w2c[kPolHidden], w2r[kPolHidden], w3[kPolArms], b3[kPolArms];
+#pragma unroll
+  for (int i = 0; i < kPolFeat; ++i) w1[i] = w[kPolOffW1 + i * kPolHidden + lane];
+#pragma unroll
+  for (int i = 0; i < kPolHidden; ++i) {
+    w2c[i] = w[kPolOffW2 + i * kPolHidden + lane];
+    w2r[i] = w[kPolOffW2 + lane * kPolHidden + i];
+  }
+#pragma unroll
+  for (int a = 0; a < kPolArms; ++a) {
+    w3[a] = w[kPolOffW3 + lane * kPolArms + a];
+    b3[a] = w[kPolOffB3 + a];
+  }
+  const float b1 = w[kPolOffB1 + lane], b2 = w[kPolOffB2 + lane];
+  float g1[kPolFeat] = {}, g2[kPolHidden] = {}, g3[kPolArms] = {}, gb1 = 0.0f, gb2 = 0.0f, gb3 = 0.0f, se = 0.0f;
+  // tiles of consecutive samples, dealt to the blocks in turn (a small batch
+  // spreads over the SMs)
+  const uint32_t tiles = (batch + kGradTile - 1) / kGradTile;
+  for (uint32_t tile = warp * gridDim.x + blockIdx.x; tile < tiles; tile += gridDim.x * kGradWarps) {
+    const uint32_t s0 = tile * kGradTile;
+    const int n = (int)min(batch - s0, (uint32_t)kGradTile);
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < kGradTile * kPolFeat / 32; ++q) {
+      const int e = q * 32 + lane;
+      (&s_x[warp][0][0])[e] = e < n * kPolFeat ? x[(size_t)s0 * kPolFeat + e] : 0.0f;
     }
-    for (int j = 0; j < kPolHidden; ++j) {
-      float z = sw[kPolOffB2 + j];
-      for (int i = 0; i < kPolHidden; ++i) z = fmaf(h1[i], sw[kPolOffW2 + i * kPolHidden + j], z);
-      z2[j] = z;
-      h2[j] = fmaxf(z, 0.0f);
+    float my_t = 0.0f;
+    uint32_t my_a = 0;
+    if (lane < n) {
+      my_t = target[s0 + lane];
+      my_a = arm[s0 + lane];
+      my_a = my_a < (uint32_t)kPolArms ? my_a : 0u;
     }
-    const uint32_t a = arm[b] < kPolArms ? arm[b] : 0;
-    float ya = sw[kPolOffB3 + a];
-    for (int i = 0; i < kPolHidden; ++i) ya = fmaf(h2[i], sw[kPolOffW3 + i * kPolArms + a], ya);
-    const float err = ya - target[b];
-    const float dya = 2.0f * err * inv_b;  // d loss / d y_b[a]
-    float* s = scr + (size_t)b * kScr;
-    float dz2[kPolHidden];
-    for (int i = 0; i < kPolHidden; ++i) dz2[i] = z2[i] > 0.0f ? sw[kPolOffW3 + i * kPolArms + a] * dya : 0.0f;
-    for (int j = 0; j < kPolHidden; ++j) {
-      float g = 0.0f;
-      for (int i = 0; i < kPolHidden; ++i) g = fmaf(sw[kPolOffW2 + j * kPolHidden + i], dz2[i], g);
-      s[kPolHidden + j] = z1[j] > 0.0f ? g : 0.0f;  // dz1
-      s[j] = h1[j];
-      s[2 * kPolHidden + j] = h2[j];
-      s[3 * kPolHidden + j] = dz2[j];
+    __syncwarp();
+    for (int s = 0; s < n; s += 2) {  // (an odd last sample's twin counts for nothing: its error is zeroed)
+      float h1[2], h2[2], g[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float z = b1;
+#pragma unroll
+        for (int i = 0; i < kPolFeat; ++i) z = fmaf(s_x[warp][s + u][i], w1[i], z);
+        h1[u] = fmaxf(z, 0.0f);
+        s_h[warp][u][lane] = h1[u];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float z = b2;
+#pragma unroll
+        for (int i = 0; i < kPolHidden; ++i) z = fmaf(s_h[warp][u][i], w2c[i], z);
+        h2[u] = fmaxf(z, 0.0f);
+      }
+      float ya[2];
+      uint32_t a[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        a[u] = __shfl_sync(0xFFFFFFFFu, my_a, s + u);
+        const float w3a = a[u] == 0 ? w3[0] : a[u] == 1 ? w3[1] : a[u] == 2 ? w3[2] : w3[3];
+        ya[u] = h2[u] * w3a;
+        g[u] = w3a;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) ya[u] += __shfl_xor_sync(0xFFFFFFFFu, ya[u], o);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float b3a = a[u] == 0 ? b3[0] : a[u] == 1 ? b3[1] : a[u] == 2 ? b3[2] : b3[3];
+        const float err = s + u < n ? ya[u] + b3a - __shfl_sync(0xFFFFFFFFu, my_t, s + u) : 0.0f;
+        const float dya = 2.0f * err * inv_b;  // d loss / d y_b[a]
+        se = fmaf(err * inv_b, err, se);
+        const float dz2 = h2[u] > 0.0f ? g[u] * dya : 0.0f;
+        g[u] = dz2;
+        s_g[warp][u][lane] = dz2;
+        gb2 += dz2;
+#pragma unroll
+        for (int k = 0; k < kPolArms; ++k) g3[k] = fmaf(h2[u], a[u] == (uint32_t)k ? dya : 0.0f, g3[k]);
+        if ((uint32_t)lane == a[u]) gb3 += dya;  // (lane k: output k)
+      }
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float d = 0.0f;
+#pragma unroll
+        for (int i = 0; i < kPolHidden; ++i) {
+          d = fmaf(w2r[i], s_g[warp][u][i], d);
+          g2[i] = fmaf(s_h[warp][u][i], g[u], g2[i]);
+        }
+        const float dz1 = h1[u] > 0.0f ? d : 0.0f;
+        gb1 += dz1;
+#pragma unroll
+        for (int i = 0; i < kPolFeat; ++i) g1[i] = fmaf(s_x[warp][s + u][i], dz1, g1[i]);
+      }
+      __syncwarp();
     }
-    for (int k = 0; k < kPolArms; ++k) s[4 * kPolHidden + k] = k == (int)a ? dya : 0.0f;
-    s[4 * kPolHidden + kPolArms] = err * err * inv_b;
+  }
+  // the upper half of the warps leave their shares, the lower half add theirs
+  for (int half = 1; half >= 0; --half) {
+    if ((warp >= kGradWarps / 2) == (half == 1)) {
+      float* row = s_grad[warp % (kGradWarps / 2)];
+      auto put = [&](int c, float v) { row[c] = half ? v : row[c] + v; };
+#pragma unroll
+      for (int i = 0; i < kPolFeat; ++i) put(kPolOffW1 + i * kPolHidden + lane, g1[i]);
+      put(kPolOffB1 + lane, gb1);
+#pragma unroll
+      for (int i = 0; i < kPolHidden; ++i) put(kPolOffW2 + i * kPolHidden + lane, g2[i]);
+      put(kPolOffB2 + lane, gb2);
+#pragma unroll
+      for (int k = 0; k < kPolArms; ++k) put(kPolOffW3 + lane * kPolArms + k, g3[k]);
+      if (lane < kPolArms) put(kPolOffB3 + lane, gb3);
+      if (lane == 0) put(kPolWeights, se);
+    }
+    __syncthreads();
+  }
+  for (int c = threadIdx.x; c < kGradRow; c += 32 * kGradWarps) {
+    float v = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kGradWarps / 2; ++q) v += s_grad[q][c];
+    partial[(size_t)blockIdx.x * kGradRow + c] = v;
   }
 }
 
-// Block r computes gradient row r.  Rows: 0..7 W1 rows (A = x[i], G = dz1),
-// 8..39 W2 rows (A = h1[i], G = dz2), 40..71 W3 rows (A = h2[i], G = dy),
-// 72 b1 (G = dz1), 73 b2 (G = dz2), 74 b3 (G = dy), 75 loss (sum of se).
-__global__ void k_mlp_grad_reduce(const float* __restrict__ x, const float* __restrict__ scr, uint32_t batch,
-                                  float* __restrict__ grad, float* __restrict__ loss) {
-  const int r = blockIdx.x;
-  int cols, gofs, outofs, aidx = -1;
-  bool ax = false;
-  if (r < 8) { ax = true; aidx = r; gofs = kPolHidden; cols = kPolHidden; outofs = kPolOffW1 + r * kPolHidden; }
-  else if (r < 40) { aidx = r - 8; gofs = 3 * kPolHidden; cols = kPolHidden; outofs = kPolOffW2 + (r - 8) * kPolHidden; }
-  else if (r < 72) { aidx = 2 * kPolHidden + (r - 40); gofs = 4 * kPolHidden; cols = kPolArms; outofs = kPolOffW3 + (r - 40) * kPolArms; }
-  else if (r == 72) { gofs = kPolHidden; cols = kPolHidden; outofs = kPolOffB1; }
-  else if (r == 73) { gofs = 3 * kPolHidden; cols = kPolHidden; outofs = kPolOffB2; }
-  else if (r == 74) { gofs = 4 * kPolHidden; cols = kPolArms; outofs = kPolOffB3; }
-  else { gofs = 4 * kPolHidden + kPolArms; cols = 1; outofs = -1; }
-  float acc[kPolHidden];
-  for (int c = 0; c < kPolHidden; ++c) acc[c] = 0.0f;
-  for (uint32_t b = threadIdx.x; b < batch; b += blockDim.x) {
-    const float* s = scr + (size_t)b * kScr;
-    const float av = aidx < 0 ? 1.0f : (ax ? x[(size_t)b * kPolFeat + aidx] : s[aidx]);
-    for (int c = 0; c < cols; ++c) acc[c] = fmaf(av, s[gofs + c], acc[c]);
+// Sums `rows` partial gradients: 32 columns a block, eight threads a column.
+__global__ void __launch_bounds__(256) k_mlp_grad_reduce(const float* __restrict__ partial, int rows,
+                                                         float* __restrict__ grad, float* __restrict__ loss) {
+  __shared__ float s[8][32];
+  const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5, c = blockIdx.x * 32 + cx;
+  float v = 0.0f;
+  if (c < kGradRow) {
+#pragma unroll 4
+    for (int r = ry; r < rows; r += 8) v += partial[(size_t)r * kGradRow + c];
   }
-  __shared__ float red[256];
-  for (int c = 0; c < cols; ++c) {
-    red[threadIdx.x] = acc[c];
-    __syncthreads();
-    for (int o = blockDim.x >> 1; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      if (outofs >= 0) grad[outofs + c] = red[0];
-      else if (loss) *loss = red[0];
-    }
-    __syncthreads();
+  s[ry][cx] = v;
+  __syncthreads();
+  if (ry == 0 && c < kGradRow) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v += s[q][cx];
+    if (c < kPolWeights) grad[c] = v;
+    else if (loss) *loss = v;
   }
 }
 
@@ -213,13 +294,14 @@ extern "C" sssp_status sssp_mlp_backward(const float* w, const float* x, const f
   clear_error();
   if (!w || !x || !target || !arm || !grad || batch == 0) return fail(SSSP_ERR_INVALID_ARG, "NULL or empty argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // one block per SM, and no more than the samples fill
+  const uint32_t tiles = (uint32_t)(((uint64_t)batch + kGradTile - 1) / kGradTile);
+  const int blocks = (int)std::min<uint32_t>(tiles, (uint32_t)sm_count());
   TmpBuf<float> sbuf(st);
-  sssp_status s = sbuf.alloc((size_t)batch * kScr);
+  sssp_status s = sbuf.alloc((size_t)blocks * kGradRow);
   if (s != SSSP_OK) return s;
-  float* scr = sbuf.p;
-  const int blocks = (int)std::min<uint32_t>((batch + 127) / 128, 1024);
-  k_mlp_samples<<<blocks, 128, 0, st>>>(w, x, target, arm, batch, scr);
-  k_mlp_grad_reduce<<<76, 256, 0, st>>>(x, scr, batch, grad, loss);
+  k_mlp_grad<<<blocks, 32 * kGradWarps, 0, st>>>(w, x, target, arm, batch, sbuf.p);
+  k_mlp_grad_reduce<<<(kGradRow + 31) / 32, 256, 0, st>>>(sbuf.p, blocks, grad, loss);
   SSSP_CUDA_TRY(cudaGetLastError());
   return SSSP_OK;
 }
