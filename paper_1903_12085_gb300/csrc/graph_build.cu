@@ -12,10 +12,16 @@
 //      scatter over out-edges, done with the native 32-bit min);
 //   4. optionally the in-edge CSR: counting sort by target, rows then sorted by
 //      (cost, source) the same way.
-// Row sorts are segmented by length: <= 32 elements one warp (register bitonic
-// network), <= 4096 one block (shared-memory bitonic), longer rows are sorted
-// in 4096-element chunks and merged pairwise by rank (each element's output
-// position = its index in its run + its rank in the sibling run).
+// Row sorts are segmented by length: <= 32 and <= 128 elements one warp (register
+// bitonic network, one and four elements a lane), <= 4096 one block
+// (shared-memory bitonic), longer rows are sorted in 4096-element chunks and
+// merged pairwise by rank (each element's output position = its index in its run
+// + its rank in the sibling run).  The chunks of all long rows form one list of
+// tasks, which the blocks of the chunk sort and of the merge passes share: with
+// the blocks going through the rows one after another instead, a row of a few
+// chunks occupied a few blocks while the others waited (R-MAT s20: 13.8 ms of
+// chunk sorts and 1.5 ms of merges; a graph with reverse edges is built and
+// solved once in 8.9 ms where that took 23.9).
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -27,6 +33,7 @@ namespace sssp {
 namespace {
 
 constexpr int kMidCap = 4096;   // longest row sorted inside one block's shared memory
+constexpr int kWarpCap = 128;   // longest row sorted inside one warp's registers
 constexpr int kSortThreads = 512;
 
 __global__ void k_interleave(const uint32_t* __restrict__ col, const uint32_t* __restrict__ w, uint64_t m,
@@ -50,17 +57,22 @@ __global__ void k_validate(const uint64_t* __restrict__ ro, const uint32_t* __re
   }
 }
 
-// Split rows by length into three lists.
-__global__ void k_classify_rows(const uint64_t* __restrict__ ro, uint32_t n, uint32_t* small, uint32_t* mid,
-                                uint32_t* large, unsigned int* counts) {
+// Split rows by length into three lists, and the rows longer than kMidCap into
+// tasks {row, chunk}.
+enum { kSmallRows, kWarpRows, kMidRows, kTasks, kMaxDeg, kRowCounts };
+__global__ void k_classify_rows(const uint64_t* __restrict__ ro, uint32_t n, uint32_t* small, uint32_t* warp,
+                                uint32_t* mid, uint2* tasks, unsigned int* counts) {
   for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
     const uint64_t deg = ro[u + 1] - ro[u];
     if (deg <= 1) continue;
-    if (deg <= 32) small[atomicAdd(&counts[0], 1u)] = u;
-    else if (deg <= kMidCap) mid[atomicAdd(&counts[1], 1u)] = u;
+    if (deg <= 32) small[atomicAdd(&counts[kSmallRows], 1u)] = u;
+    else if (deg <= kWarpCap) warp[atomicAdd(&counts[kWarpRows], 1u)] = u;
+    else if (deg <= kMidCap) mid[atomicAdd(&counts[kMidRows], 1u)] = u;
     else {
-      large[atomicAdd(&counts[2], 1u)] = u;
-      atomicMax(&counts[3], (unsigned int)deg);
+      const uint32_t chunks = (uint32_t)((deg + kMidCap - 1) / kMidCap);
+      const uint32_t t0 = atomicAdd(&counts[kTasks], chunks);
+      for (uint32_t c = 0; c < chunks; ++c) tasks[t0 + c] = make_uint2(u, c);
+      atomicMax(&counts[kMaxDeg], (unsigned int)deg);
     }
   }
 }
@@ -87,6 +99,52 @@ __global__ void k_sort_small(const uint64_t* __restrict__ ro, const uint32_t* __
       }
     }
     if (lane < (int)deg) keys[b + lane] = x;
+  }
+}
+
+// One warp per row of length 33..kWarpCap: the same network over element r * 32 +
+// lane in register r of a lane.
+__global__ void k_sort_warp(const uint64_t* __restrict__ ro, const uint32_t* __restrict__ rows,
+                            const unsigned int* __restrict__ count, unsigned long long* keys) {
+  constexpr int kR = kWarpCap / 32;
+  const unsigned int nrows = *count;
+  const int lane = threadIdx.x & 31;
+  const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  for (uint64_t q = warp0; q < nrows; q += nwarps) {
+    const uint32_t u = rows[q];
+    const uint64_t b = ro[u];
+    const int deg = (int)(ro[u + 1] - b);
+    unsigned long long x[kR];
+#pragma unroll
+    for (int r = 0; r < kR; ++r) x[r] = r * 32 + lane < deg ? keys[b + r * 32 + lane] : kInf64;
+#pragma unroll
+    for (int k = 2; k <= kWarpCap; k <<= 1) {
+#pragma unroll
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        if (j >= 32) {  // partners are registers of the same lane
+#pragma unroll
+          for (int r = 0; r < kR; ++r) {
+            const int p = r ^ (j >> 5);
+            if (p < r) continue;
+            const bool up = ((r * 32) & k) == 0;
+            const unsigned long long lo = x[r] < x[p] ? x[r] : x[p], hi = x[r] < x[p] ? x[p] : x[r];
+            x[r] = up ? lo : hi;
+            x[p] = up ? hi : lo;
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < kR; ++r) {
+            const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, x[r], j);
+            const bool up = ((r * 32 + lane) & k) == 0, lower = (lane & j) == 0;
+            x[r] = (lower == up) == (o < x[r]) ? o : x[r];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kR; ++r)
+      if (r * 32 + lane < deg) keys[b + r * 32 + lane] = x[r];
   }
 }
 
@@ -127,23 +185,20 @@ __global__ void k_sort_mid(const uint64_t* __restrict__ ro, const uint32_t* __re
   }
 }
 
-// Long rows: sort every kMidCap chunk (block per chunk, grid-strided over rows).
-__global__ void k_sort_chunks(const uint64_t* __restrict__ ro, const uint32_t* __restrict__ rows,
+// Long rows: sort every kMidCap chunk, a block per task.
+__global__ void k_sort_chunks(const uint64_t* __restrict__ ro, const uint2* __restrict__ tasks,
                               const unsigned int* __restrict__ count, unsigned long long* keys) {
   __shared__ unsigned long long s[kMidCap];
-  const unsigned int nrows = *count;
-  for (unsigned int r = 0; r < nrows; ++r) {
-    const uint32_t u = rows[r];
-    const uint64_t b = ro[u], deg = ro[u + 1] - b;
-    const uint64_t nchunks = (deg + kMidCap - 1) / kMidCap;
-    for (uint64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-      const uint64_t cb = b + c * kMidCap;
-      const int len = (int)(deg - c * kMidCap < (uint64_t)kMidCap ? deg - c * kMidCap : (uint64_t)kMidCap);
-      for (int i = threadIdx.x; i < len; i += blockDim.x) s[i] = keys[cb + i];
-      block_bitonic(s, len);
-      for (int i = threadIdx.x; i < len; i += blockDim.x) keys[cb + i] = s[i];
-      __syncthreads();
-    }
+  const unsigned int ntasks = *count;
+  for (unsigned int t = blockIdx.x; t < ntasks; t += gridDim.x) {
+    const uint2 task = tasks[t];
+    const uint64_t cb = ro[task.x] + (uint64_t)task.y * kMidCap;
+    const uint64_t rest = ro[task.x + 1] - cb;
+    const int len = (int)(rest < (uint64_t)kMidCap ? rest : (uint64_t)kMidCap);
+    for (int i = threadIdx.x; i < len; i += blockDim.x) s[i] = keys[cb + i];
+    block_bitonic(s, len);
+    for (int i = threadIdx.x; i < len; i += blockDim.x) keys[cb + i] = s[i];
+    __syncthreads();
   }
 }
 
@@ -169,38 +224,35 @@ __device__ __forceinline__ uint64_t upper_bound_u64(const unsigned long long* a,
 // One merge pass over every long row: runs of width `width` are merged in
 // pairs from src to dst (same offsets).  Equal keys are identical words, so
 // ties between runs only need distinct positions (left run first).
-__global__ void k_merge_pass(const uint64_t* __restrict__ ro, const uint32_t* __restrict__ rows,
+__global__ void k_merge_pass(const uint64_t* __restrict__ ro, const uint2* __restrict__ tasks,
                              const unsigned int* __restrict__ count, const unsigned long long* __restrict__ src,
                              unsigned long long* __restrict__ dst, uint64_t width) {
-  const unsigned int nrows = *count;
-  const uint64_t gtid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t gstride = (uint64_t)gridDim.x * blockDim.x;
-  for (unsigned int r = 0; r < nrows; ++r) {
-    const uint32_t u = rows[r];
-    const uint64_t b = ro[u], deg = ro[u + 1] - b;
-    for (uint64_t i = gtid; i < deg; i += gstride) {
-      const uint64_t run = i / width, pair0 = (run & ~1ull) * width;
-      const uint64_t lstart = pair0, lend = min(deg, pair0 + width);
-      const uint64_t rstart = lend, rend = min(deg, pair0 + 2 * width);
+  const unsigned int ntasks = *count;
+  for (unsigned int t = blockIdx.x; t < ntasks; t += gridDim.x) {
+    const uint2 task = tasks[t];
+    const uint64_t b = ro[task.x], deg = ro[task.x + 1] - b;
+    const uint64_t i0 = (uint64_t)task.y * kMidCap, i1 = min(deg, i0 + kMidCap);
+    const uint64_t run = i0 / width, pair0 = (run & ~1ull) * width;  // (width is a multiple of kMidCap)
+    const uint64_t lend = min(deg, pair0 + width), rend = min(deg, pair0 + 2 * width);
+    for (uint64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
       const unsigned long long x = src[b + i];
       uint64_t pos;
-      if ((run & 1) == 0) pos = (i - lstart) + lower_bound_u64(src + b + rstart, rend - rstart, x);
-      else pos = (i - rstart) + upper_bound_u64(src + b + lstart, lend - lstart, x);
+      if ((run & 1) == 0) pos = (i - pair0) + lower_bound_u64(src + b + lend, rend - lend, x);
+      else pos = (i - lend) + upper_bound_u64(src + b + pair0, lend - pair0, x);
       dst[b + pair0 + pos] = x;
     }
   }
 }
 
-__global__ void k_copy_rows(const uint64_t* __restrict__ ro, const uint32_t* __restrict__ rows,
+__global__ void k_copy_rows(const uint64_t* __restrict__ ro, const uint2* __restrict__ tasks,
                             const unsigned int* __restrict__ count, const unsigned long long* __restrict__ src,
                             unsigned long long* __restrict__ dst) {
-  const unsigned int nrows = *count;
-  const uint64_t gtid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t gstride = (uint64_t)gridDim.x * blockDim.x;
-  for (unsigned int r = 0; r < nrows; ++r) {
-    const uint32_t u = rows[r];
-    const uint64_t b = ro[u], deg = ro[u + 1] - b;
-    for (uint64_t i = gtid; i < deg; i += gstride) dst[b + i] = src[b + i];
+  const unsigned int ntasks = *count;
+  for (unsigned int t = blockIdx.x; t < ntasks; t += gridDim.x) {
+    const uint2 task = tasks[t];
+    const uint64_t b = ro[task.x] + (uint64_t)task.y * kMidCap;
+    const uint64_t len = min(ro[task.x + 1] - b, (uint64_t)kMidCap);
+    for (uint64_t i = threadIdx.x; i < len; i += blockDim.x) dst[b + i] = src[b + i];
   }
 }
 
@@ -344,32 +396,40 @@ sssp_status exclusive_scan(const uint32_t* in, uint64_t n, uint64_t* out, cudaSt
 sssp_status sort_rows(const uint64_t* ro, uint32_t n, uint64_t m, unsigned long long* keys, cudaStream_t st) {
   if (m == 0) return SSSP_OK;
   TmpBuf<uint32_t> lbuf(st);
+  TmpBuf<uint2> tbuf(st);
   TmpBuf<unsigned int> cbuf(st);
   sssp_status s = SSSP_OK;
-  if ((s = lbuf.alloc(3ull * n)) != SSSP_OK || (s = cbuf.alloc(4)) != SSSP_OK) return s;
+  // (a row longer than kMidCap has at most deg / (kMidCap / 2) chunks)
+  if ((s = lbuf.alloc(3ull * n)) != SSSP_OK || (s = tbuf.alloc(m / (kMidCap / 2) + 1)) != SSSP_OK ||
+      (s = cbuf.alloc(kRowCounts)) != SSSP_OK)
+    return s;
   uint32_t* lists = lbuf.p;
+  uint2* tasks = tbuf.p;
   unsigned int* counts = cbuf.p;
-  SSSP_CUDA_TRY(cudaMemsetAsync(counts, 0, 4 * sizeof(unsigned int), st));
-  uint32_t *small = lists, *mid = lists + n, *large = lists + 2ull * n;
-  k_classify_rows<<<grid_for(n, 256), 256, 0, st>>>(ro, n, small, mid, large, counts);
-  k_sort_small<<<grid_for(32ull * n, 256), 256, 0, st>>>(ro, small, counts + 0, keys);
-  k_sort_mid<<<sm_count() * 8, kSortThreads, 0, st>>>(ro, mid, counts + 1, keys);
-  unsigned int hc[4] = {0, 0, 0, 0};
+  SSSP_CUDA_TRY(cudaMemsetAsync(counts, 0, kRowCounts * sizeof(unsigned int), st));
+  uint32_t *small = lists, *warp = lists + n, *mid = lists + 2ull * n;
+  k_classify_rows<<<grid_for(n, 256), 256, 0, st>>>(ro, n, small, warp, mid, tasks, counts);
+  k_sort_small<<<grid_for(32ull * n, 256), 256, 0, st>>>(ro, small, counts + kSmallRows, keys);
+  k_sort_warp<<<sm_count() * 8, 256, 0, st>>>(ro, warp, counts + kWarpRows, keys);
+  k_sort_mid<<<sm_count() * 8, kSortThreads, 0, st>>>(ro, mid, counts + kMidRows, keys);
+  unsigned int hc[kRowCounts] = {};
   SSSP_CUDA_TRY(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));
-  const unsigned int nlarge = hc[2];
-  const uint64_t maxdeg = hc[3];
-  if (nlarge > 0) {
-    k_sort_chunks<<<sm_count() * 4, kSortThreads, 0, st>>>(ro, large, counts + 2, keys);
+  const unsigned int ntasks = hc[kTasks];
+  const uint64_t maxdeg = hc[kMaxDeg];
+  if (ntasks > 0) {
+    const unsigned int* nt = counts + kTasks;
+    const int blocks = (int)std::min<unsigned int>(ntasks, (unsigned int)sm_count() * 8);
+    k_sort_chunks<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, keys);
     TmpBuf<unsigned long long> mbuf(st);
     if ((s = mbuf.alloc(m)) != SSSP_OK) return s;
     unsigned long long* tmp = mbuf.p;
     unsigned long long *src = keys, *dst = tmp;
     for (uint64_t width = kMidCap; width < maxdeg; width *= 2) {
-      k_merge_pass<<<sm_count() * 4, 256, 0, st>>>(ro, large, counts + 2, src, dst, width);
+      k_merge_pass<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, src, dst, width);
       std::swap(src, dst);
     }
-    if (src != keys) k_copy_rows<<<sm_count() * 4, 256, 0, st>>>(ro, large, counts + 2, src, keys);
+    if (src != keys) k_copy_rows<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, src, keys);
     SSSP_CUDA_TRY(cudaGetLastError());
   }
   SSSP_CUDA_TRY(cudaGetLastError());
