@@ -1213,7 +1213,7 @@ __device__ __forceinline__ bool run_phase(bool alone, uint64_t k, uint32_t nf_co
 // settled, 124 edges) a phase takes 3.3 us; with the fringe as a queue of
 // vertices, whose records, settled rows, edges, targets and claims were five
 // round trips and whose scan was bound by one SM's gathers, it took 6.0 us
-// (206 -> 114 ms a solve; 256 sources on the 512 x 512 grid 117 -> 72 ms).
+// (206 -> 112 ms a solve; 256 sources on the 512 x 512 grid 117 -> 72 ms).
 //
 // Entry: global queue q[(k-1)&1] with slot[k%4].qcount entries, thresholds in
 // slot[k%4].  Exit at phase k: the same state with slot[(k+1)%4] reset, or
@@ -1412,15 +1412,17 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     minD = (T)(d - base);
     minOut = o - base > inf ? inf : (T)(o - base);
   }
-  unsigned int since_pick = s_solo_cont ? s_solo_since : 0u;
-  Arm arm = s_solo_cont ? s_solo_arm : Arm{false, false, -1};
-  // counters of the last phase (policy features), and of the episode
-  uint32_t e_prev = 0, s_prev = 0, f_prev = 0;
-  if (kKind != kStatic) {
-    e_prev = (uint32_t)ldcg_u64(&ctl->slot[(k + 3) % 4].relax_packed);
-    s_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].settled_now);
-    f_prev = ldcg_u32(&ctl->slot[(k + 3) % 4].fsize);
+  // The arm (s_solo_arm) is chosen in phase `pick`: the policy's in the first phase
+  // of the episode and every 8th after it (the choice is logged per phase either way).
+  uint32_t pick = k;
+  bool in_dyn = false;
+  if (kKind != kStatic && s_solo_cont) {
+    const uint32_t since = s_solo_since;
+    pick = !policy ? kInf32 : since ? k + 8 - since : k;
+    in_dyn = s_solo_arm.in_simple && use_in && w.cur_in != nullptr;
   }
+  const uint32_t k_first = k;
+  // counters of the episode
   unsigned long long sum_f = 0, sum_s = 0, sum_e = 0;
   if (tid == 0) solo_clear(&s_sc[k & 1]);
   uint32_t live = 0, spent = 0;  // this thread's fringe slots / those it settled in the last phase
@@ -1455,17 +1457,27 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
 
   for (;;) {
     SoloCount* const sc = &s_sc[k & 1];
-    // the policy is evaluated on the first phase of the episode and every 8th
-    // phase after it (the choice is logged per phase either way)
-    if (kKind != kStatic && SSSP_RARE(since_pick == 0)) {
-      arm = choose_arm(p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
-      if (tid == 0) s_solo_arm = arm;
+    if (kKind != kStatic && SSSP_RARE(k == pick)) {
+      uint32_t e_prev, s_prev, f_prev;  // counters of the last phase
+      if (k == k_first) {
+        const PhaseSlot* Sp = &ctl->slot[(k + 3) % 4];
+        e_prev = (uint32_t)ldcg_u64(&Sp->relax_packed);
+        s_prev = ldcg_u32(&Sp->settled_now);
+        f_prev = ldcg_u32(&Sp->fsize);
+      } else {
+        const SoloCount* sp = &s_sc[(k + 1) & 1];
+        e_prev = sp->edges;
+        s_prev = sp->settled;
+        f_prev = nF + s_prev - sp->fresh + (kNF ? far - (uint32_t)sp->far : 0u);
+      }
+      const Arm arm = choose_arm(p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
+      if (tid == 0) s_solo_arm = arm;  // (read past a barrier)
+      pick = policy ? k + 8 : kInf32;
+      in_dyn = arm.in_simple && use_in && w.cur_in != nullptr;
     }
-    since_pick = policy ? (since_pick + 1) & 7u : 1u;
-    const bool in_dyn = kKind != kStatic && arm.in_simple && use_in && w.cur_in != nullptr;
     if (scribe && trace) s_t0 = globaltimer_ns();
     live = m.used[tid] & ~spent;
-    if (SSSP_RARE(in_dyn || was_dyn)) {  // minima of this phase's variant (IN-SIMPLE reads status bytes the selection writes)
+    if (kKind != kStatic && SSSP_RARE(in_dyn || was_dyn)) {  // minima of this phase's variant (IN-SIMPLE reads status bytes the selection writes)
       // (the warp's slots in use, dealt to its lanes evenly: a cursor's round
       // trips follow one another)
       uint8_t* ids = reinterpret_cast<uint8_t*>(m.list);
@@ -1752,9 +1764,6 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     sum_f += fs;
     sum_s += settled_now;
     sum_e += E;
-    e_prev = E;
-    s_prev = settled_now;
-    f_prev = fs;
     if (tid == 0) ctl->heartbeat = k;
     if (trace && scribe && k <= w.trace_cap) {
       sssp_phase_record r;
@@ -1766,7 +1775,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
       uint32_t c = p.crit & SSSP_CRITERIA_MASK;
       if (use_in) c = (c & ~(uint32_t)(SSSP_IN_STATIC | SSSP_IN_SIMPLE)) | (in_dyn ? SSSP_IN_SIMPLE : SSSP_IN_STATIC);
       r.criterion = c;
-      r.arm = arm_code(arm, true) | nf_code;
+      r.arm = arm_code(s_solo_arm, true) | nf_code;
       r.t_start_ns = s_t0;
       r.t_end_ns = globaltimer_ns();
       r.queued = nF;
@@ -1793,11 +1802,11 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     s_st.relaxed += sum_e;
   }
   if (hand) {
-    if (tid == 0) s_solo_arm = arm;
+    if (kKind == kStatic && tid == 0) s_solo_arm = Arm{false, false, -1};
     solo_hand_off<T>(k, live & ~sel, sel, od, oo, base, minD, minOut, nF, far, nf_code, s_t0);
     if (tid == 0 && (!group || (uint32_t)s_solo_n <= p.solo_edges)) {
       s_solo_cont = 1;
-      s_solo_since = since_pick;
+      s_solo_since = policy ? (k + 9 - pick) & 7u : 1u;
     }
     __threadfence();
     __syncthreads();
@@ -1816,9 +1825,10 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     if (minD != inf) S0->min_d = base + minD;
     if (minOut != inf) S0->min_out = base + minOut;
     PhaseSlot* Sp = &ctl->slot[(k + 3) % 4];  // the last solo phase, for the policy's features
-    Sp->relax_packed = e_prev;
-    Sp->settled_now = s_prev;
-    Sp->fsize = f_prev;
+    const SoloCount* sp = &s_sc[(k + 1) & 1];
+    Sp->relax_packed = sp->edges;
+    Sp->settled_now = sp->settled;
+    Sp->fsize = nF + sp->settled - sp->fresh + (kNF ? far - (uint32_t)sp->far : 0u);
   }
   __threadfence();
   __syncthreads();
@@ -2634,6 +2644,17 @@ __global__ void __launch_bounds__(kT, kThreads / kT) k_solve_batch(const BatchIt
 // ---------------------------------------------------------------------------
 // host side
 
+// Graphs of at most kSoloLargeN vertices, or with fewer than 6 edges a vertex
+// (meshes and the like, whose fringes stay small for many phases), get twice the
+// slots: their solves live in episodes.  On larger and denser ones the grid
+// phases count, and these want the L1 that the slots would take.  (G(2^14, 2^17)
+// with 4, 8, 12, 16 slots a thread: 1.47, 1.37, 1.43, 1.64 ms; the 1024 x 1024
+// grid 110.7, 108.9, 110.4, 110.3.)  In blocks of kSmallThreads, two to an SM,
+// the meshes alone: 200 solves of G(20000, 160000) take 5.5 ms with 16 slots a
+// thread, 4.2 with 8, and 256 sources on the 512 x 512 grid 48 and 73.
+static bool solo_mesh(uint32_t n, uint64_t m) { return m < 6ull * n; }
+static bool solo_large(uint32_t n, uint64_t m) { return n <= kSoloLargeN || solo_mesh(n, m); }
+
 // The kernel instance for a criterion mask (see kAny).
 int kind_of(uint32_t crit, bool narrow, bool records) {
   constexpr uint32_t is = SSSP_IN_STATIC | SSSP_OUT_STATIC;
@@ -2751,17 +2772,6 @@ size_t solo_shape_of(bool large, bool narrow, uint32_t crit, uint32_t threads, P
   p->pol_off = (uint32_t)((std::max(kGridSmem, solo) + 15) / 16 * 16);
   return p->pol_off + (policy ? kPolicySmem : 0);
 }
-
-// Graphs of at most kSoloLargeN vertices, or with fewer than 6 edges a vertex
-// (meshes and the like, whose fringes stay small for many phases), get twice the
-// slots: their solves live in episodes.  On larger and denser ones the grid
-// phases count, and these want the L1 that the slots would take.  (G(2^14, 2^17)
-// with 4, 8, 12, 16 slots a thread: 1.47, 1.37, 1.43, 1.64 ms; the 1024 x 1024
-// grid 110.7, 108.9, 110.4, 110.3.)  In blocks of kSmallThreads, two to an SM,
-// the meshes alone: 200 solves of G(20000, 160000) take 5.5 ms with 16 slots a
-// thread, 4.2 with 8, and 256 sources on the 512 x 512 grid 48 and 73.
-bool solo_mesh(uint32_t n, uint64_t m) { return m < 6ull * n; }
-bool solo_large(uint32_t n, uint64_t m) { return n <= kSoloLargeN || solo_mesh(n, m); }
 
 }  // namespace
 
@@ -2937,7 +2947,11 @@ struct BatchPlan {
   uint32_t crit = 0;
   bool large = true, mesh = true, narrow = true;  // see solo_shape_of
   uint32_t recording = 0;              // solves with a trace or settle phases attached
-  int kind() const { return kind_of(crit, narrow, recording != 0); }
+  // Policy solves of graphs with small episodes (solo_large) run mostly grid
+  // phases, whose steps spill least in the batch's general instance: 8 sources of
+  // G(2^24, 2^28) at once 119 ms, in the instance for the arms 121.4.  (Single
+  // solves are the other way round: G(2^20, 2^24) 8.6 and 8.2 ms.)
+  int kind() const { return kind_of(crit, narrow, recording != 0 || (!large && (crit & SSSP_POLICY_LEARNED))); }
   uint32_t bpg = 1;                    // blocks per solve
   bool staged = false;                 // bpg = 1: larger solves get more blocks
   uint32_t slots = 0;                  // gslots allocated (any stages fit)
