@@ -195,12 +195,13 @@ k_mlp_grad(const float* __restrict__ w, const float* __restrict__ x, const float
   }
 }
 
-// Sums `rows` partial gradients: 32 columns a block, eight threads a column.
+// Sums `rows` partial gradients: 32 columns a block, eight threads a column, in
+// 64 bits (19 additions a thread), so that the sum's own error does not count.
 __global__ void __launch_bounds__(256) k_mlp_grad_reduce(const float* __restrict__ partial, int rows,
                                                          float* __restrict__ grad, float* __restrict__ loss) {
-  __shared__ float s[8][32];
+  __shared__ double s[8][32];
   const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5, c = blockIdx.x * 32 + cx;
-  float v = 0.0f;
+  double v = 0.0;
   if (c < kGradRow) {
 #pragma unroll 4
     for (int r = ry; r < rows; r += 8) v += partial[(size_t)r * kGradRow + c];
@@ -210,8 +211,8 @@ __global__ void __launch_bounds__(256) k_mlp_grad_reduce(const float* __restrict
   if (ry == 0 && c < kGradRow) {
 #pragma unroll
     for (int q = 1; q < 8; ++q) v += s[q][cx];
-    if (c < kPolWeights) grad[c] = v;
-    else if (loss) *loss = v;
+    if (c < kPolWeights) grad[c] = (float)v;
+    else if (loss) *loss = (float)v;
   }
 }
 
