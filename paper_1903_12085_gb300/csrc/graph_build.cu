@@ -35,6 +35,7 @@ namespace {
 constexpr int kMidCap = 4096;   // longest row sorted inside one block's shared memory
 constexpr int kWarpCap = 128;   // longest row sorted inside one warp's registers
 constexpr int kSortThreads = 512;
+constexpr int kMergeParts = kMidCap / kSortThreads;  // blocks that share a task's merge
 
 __global__ void k_interleave(const uint32_t* __restrict__ col, const uint32_t* __restrict__ w, uint64_t m,
                              unsigned long long* __restrict__ keys) {
@@ -221,20 +222,21 @@ __device__ __forceinline__ uint64_t upper_bound_u64(const unsigned long long* a,
   return lo;
 }
 
-// One merge pass over every long row: runs of width `width` are merged in
-// pairs from src to dst (same offsets).  Equal keys are identical words, so
+// One merge pass over every long row: runs of width `width` are merged in pairs
+// from src to dst (same offsets), a thread per element and a task in kMergeParts
+// blocks (a thread's searches are chains of dependent loads).  Equal keys are identical words, so
 // ties between runs only need distinct positions (left run first).
 __global__ void k_merge_pass(const uint64_t* __restrict__ ro, const uint2* __restrict__ tasks,
                              const unsigned int* __restrict__ count, const unsigned long long* __restrict__ src,
                              unsigned long long* __restrict__ dst, uint64_t width) {
-  const unsigned int ntasks = *count;
-  for (unsigned int t = blockIdx.x; t < ntasks; t += gridDim.x) {
-    const uint2 task = tasks[t];
+  const uint64_t nparts = (uint64_t)*count * kMergeParts;
+  for (uint64_t t = blockIdx.x; t < nparts; t += gridDim.x) {
+    const uint2 task = tasks[t / kMergeParts];
     const uint64_t b = ro[task.x], deg = ro[task.x + 1] - b;
-    const uint64_t i0 = (uint64_t)task.y * kMidCap, i1 = min(deg, i0 + kMidCap);
-    const uint64_t run = i0 / width, pair0 = (run & ~1ull) * width;  // (width is a multiple of kMidCap)
+    const uint64_t i = (uint64_t)task.y * kMidCap + t % kMergeParts * kSortThreads + threadIdx.x;
+    const uint64_t run = i / width, pair0 = (run & ~1ull) * width;
     const uint64_t lend = min(deg, pair0 + width), rend = min(deg, pair0 + 2 * width);
-    for (uint64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    if (i < deg) {
       const unsigned long long x = src[b + i];
       uint64_t pos;
       if ((run & 1) == 0) pos = (i - pair0) + lower_bound_u64(src + b + lend, rend - lend, x);
@@ -247,12 +249,11 @@ __global__ void k_merge_pass(const uint64_t* __restrict__ ro, const uint2* __res
 __global__ void k_copy_rows(const uint64_t* __restrict__ ro, const uint2* __restrict__ tasks,
                             const unsigned int* __restrict__ count, const unsigned long long* __restrict__ src,
                             unsigned long long* __restrict__ dst) {
-  const unsigned int ntasks = *count;
-  for (unsigned int t = blockIdx.x; t < ntasks; t += gridDim.x) {
-    const uint2 task = tasks[t];
-    const uint64_t b = ro[task.x] + (uint64_t)task.y * kMidCap;
-    const uint64_t len = min(ro[task.x + 1] - b, (uint64_t)kMidCap);
-    for (uint64_t i = threadIdx.x; i < len; i += blockDim.x) dst[b + i] = src[b + i];
+  const uint64_t nparts = (uint64_t)*count * kMergeParts;
+  for (uint64_t t = blockIdx.x; t < nparts; t += gridDim.x) {
+    const uint2 task = tasks[t / kMergeParts];
+    const uint64_t i = ro[task.x] + (uint64_t)task.y * kMidCap + t % kMergeParts * kSortThreads + threadIdx.x;
+    if (i < ro[task.x + 1]) dst[i] = src[i];
   }
 }
 
@@ -419,17 +420,18 @@ sssp_status sort_rows(const uint64_t* ro, uint32_t n, uint64_t m, unsigned long 
   const uint64_t maxdeg = hc[kMaxDeg];
   if (ntasks > 0) {
     const unsigned int* nt = counts + kTasks;
-    const int blocks = (int)std::min<unsigned int>(ntasks, (unsigned int)sm_count() * 8);
+    const int blocks = (int)std::min<uint64_t>(ntasks, (uint64_t)sm_count() * 8);
+    const int parts = (int)std::min<uint64_t>((uint64_t)ntasks * kMergeParts, (uint64_t)sm_count() * 8);
     k_sort_chunks<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, keys);
     TmpBuf<unsigned long long> mbuf(st);
     if ((s = mbuf.alloc(m)) != SSSP_OK) return s;
     unsigned long long* tmp = mbuf.p;
     unsigned long long *src = keys, *dst = tmp;
     for (uint64_t width = kMidCap; width < maxdeg; width *= 2) {
-      k_merge_pass<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, src, dst, width);
+      k_merge_pass<<<parts, kSortThreads, 0, st>>>(ro, tasks, nt, src, dst, width);
       std::swap(src, dst);
     }
-    if (src != keys) k_copy_rows<<<blocks, kSortThreads, 0, st>>>(ro, tasks, nt, src, keys);
+    if (src != keys) k_copy_rows<<<parts, kSortThreads, 0, st>>>(ro, tasks, nt, src, keys);
     SSSP_CUDA_TRY(cudaGetLastError());
   }
   SSSP_CUDA_TRY(cudaGetLastError());
