@@ -113,7 +113,7 @@ struct Ctl {
   int err;                  // sssp_status recorded by a device-side failure
   unsigned int gate;        // solo mode: bumped when the leader hands back to the group
   unsigned long long heartbeat;  // solo mode: phases done by the leader (progress for waiters)
-  unsigned long long next_phase; // solo mode: 2 k + 1 if the group resumes at the relax step of phase k, 2 k at its start
+  unsigned long long next_phase; // solo mode: 4 k, phase the group goes on with, + kSoloResume or kSoloNoFit (see solo_episode)
   GridBarrier bar;
   // near/far split: far fringe vertices, a work counter and two key
   // histograms (use u fills hist[u & 1] while the other one is cleared)
@@ -127,6 +127,9 @@ struct Ctl {
   unsigned int nf_beyond;
   unsigned int nf_moved;  // vertices a pull moved to the queue (summed before the far count drops)
   unsigned int nf_cnt[kNfRing];
+  // solo mode: blocks that have decided to wait for an episode (size - 1 more
+  // with every episode), see episode_join
+  unsigned int arrived;
 };
 
 // Mutable per-solve buffers.
@@ -325,6 +328,23 @@ __device__ __forceinline__ bool bounded_wait_change(const unsigned int* addr, un
         if (p != last) { last = p; t0 = now; }
       }
       if (now - t0 > limit_ns) {
+        atomicCAS(err, 0, (int)SSSP_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// Spin until *addr == want, with the same limits.
+__device__ __forceinline__ bool bounded_wait_value(const unsigned int* addr, unsigned int want,
+                                                   unsigned long long limit_ns, int* err) {
+  const unsigned long long t0 = globaltimer_ns();
+  unsigned int spins = 0;
+  while (ld_acquire_gpu(addr) != want) {
+    if ((++spins & 15u) == 0) {
+      if (*(volatile int*)err != 0) return false;
+      if (globaltimer_ns() - t0 > limit_ns) {
         atomicCAS(err, 0, (int)SSSP_ERR_TIMEOUT);
         return false;
       }

@@ -406,6 +406,18 @@ static __shared__ Mode s_md;
 static __shared__ Stats s_st;
 static __shared__ NfView s_nv;
 static __shared__ uint32_t s_nf_uses;  // key histograms used so far
+static __shared__ uint32_t s_arrivals;  // leading block: what ctl->arrived is once every block waits
+
+// Every block decides from the phase's head (load_head) whether an episode
+// begins, and the leading block rewrites those words when it leaves the
+// episode.  So the others say that they have decided (episode_wait), and one
+// thread of the leading block waits for them here before the first barrier of
+// the episode, beside the loads of the fringe.  (If the wait runs out the
+// error is recorded, and the group's next wait ends the solve.)
+__device__ __noinline__ void episode_join() {
+  s_arrivals += s_grp.size - 1;
+  bounded_wait_value(&s_p.ws.ctl->arrived, s_arrivals, s_grp.limit, s_grp.err);
+}
 
 // Bucket of a far vertex's stored word (key > B >= O).
 __device__ __forceinline__ uint32_t nf_bucket(const NfView& nv, unsigned long long word, uint32_t im) {
@@ -1390,7 +1402,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
   const uint2* const rowdeg = p.g.rowdeg;
   const unsigned int tid = threadIdx.x, nthr = blockDim.x;
   const unsigned int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
-  const bool scribe = tid == nthr - 32;  // writes the trace
+  const bool scribe = tid == nthr - 32;  // writes the trace, waits for the group
   const uint32_t spt = p.solo_spt;       // slots per thread (at most 16)
   const bool use_in = s_md.use_in, use_out = s_md.use_out;
   uint8_t* const status = kKind != kStatic && status_live(s_md, kNF) ? w.status : nullptr;
@@ -1426,6 +1438,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
   unsigned long long sum_f = 0, sum_s = 0, sum_e = 0;
   if (tid == 0) solo_clear(&s_sc[k & 1]);
   uint32_t live = 0, spent = 0;  // this thread's fringe slots / those it settled in the last phase
+  if (group && scribe) episode_join();  // (the warp with the fewest slots to load)
   {
     const uint32_t* gq = w.q[(k - 1) & 1];
     bool fits = true;
@@ -2332,6 +2345,7 @@ __device__ __noinline__ bool solve_init(const Grp grp_in) {
     s_arm_k = ~0ull;
     s_solo_cont = 0;
     s_nf_uses = 0;
+    s_arrivals = 0;
     s_nv.bound = kNoBound;
     s_nv.origin = 0;
     s_nv.shift = 0;
@@ -2396,6 +2410,9 @@ __device__ __noinline__ uint64_t generic_solo(uint64_t k) {
   const SolveParams& p = s_p;
   Ctl* const ctl = p.ws.ctl;
   PhaseHead h = load_head(ctl, k, false);
+  // (ordered by the barriers of phase k; the queue length, all that the others
+  // read of the head for these criteria, is reset in phase k + 2)
+  if (threadIdx.x == blockDim.x - 32) episode_join();
   while (h.nQ != 0 && h.nQ <= p.solo_max && k <= (uint64_t)p.g.n + 1) {
     run_phase<kAny>(true, k, 0u, h);
     ++k;
@@ -2406,7 +2423,8 @@ __device__ __noinline__ uint64_t generic_solo(uint64_t k) {
 }
 
 // The leading block's word to the group after an episode, and the others' wait
-// for it (0 if the wait ran out): what solo_episode returned.
+// for it (0 if the wait ran out): what solo_episode returned.  The barrier in
+// front of the arrival: all threads of the block have read the phase's head.
 __device__ __noinline__ void episode_end(uint64_t r) {
   Ctl* const ctl = s_p.ws.ctl;
   __syncthreads();
@@ -2420,7 +2438,9 @@ __device__ __noinline__ void episode_end(uint64_t r) {
 __device__ __noinline__ uint64_t episode_wait(unsigned int episodes) {
   __shared__ unsigned long long s_next;
   Ctl* const ctl = s_p.ws.ctl;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    red_release_gpu_add(&ctl->arrived, 1u);
     const bool ok = bounded_wait_change(&ctl->gate, episodes, s_grp.limit, s_grp.err, &ctl->heartbeat);
     s_next = ok ? ld_relaxed_gpu_u64(&ctl->next_phase) : 0ull;
   }
