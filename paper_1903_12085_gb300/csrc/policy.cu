@@ -55,6 +55,8 @@ __global__ void k_mlp_forward(const float* __restrict__ w, const float* __restri
 constexpr int kGradRow = kPolWeights + 1;
 constexpr int kGradWarps = 8;
 constexpr int kGradTile = 8;  // samples a warp takes at a time
+__host__ __device__ constexpr uint32_t grad_tiles(uint32_t batch) { return batch / kGradTile + (batch % kGradTile != 0); }
+static_assert(grad_tiles(~0u) == 1u << 29 && grad_tiles(9) == 2 && grad_tiles(8) == 1, "no wrap-around");
 
 // Gradient of the batch, one partial gradient per block.  Bound by the FP32
 // pipes and the latency of a sample's chain (about 115 multiply-adds a lane and
@@ -88,7 +90,7 @@ k_mlp_grad(const float* __restrict__ w, const float* __restrict__ x, const float
   float g1[kPolFeat] = {}, g2[kPolHidden] = {}, g3[kPolArms] = {}, gb1 = 0.0f, gb2 = 0.0f, gb3 = 0.0f, se = 0.0f;
   // tiles of consecutive samples, dealt to the blocks in turn (a small batch
   // spreads over the SMs)
-  const uint32_t tiles = (batch + kGradTile - 1) / kGradTile;
+  const uint32_t tiles = grad_tiles(batch);
   for (uint32_t tile = warp * gridDim.x + blockIdx.x; tile < tiles; tile += gridDim.x * kGradWarps) {
     const uint32_t s0 = tile * kGradTile;
     const int n = (int)min(batch - s0, (uint32_t)kGradTile);
@@ -296,8 +298,7 @@ extern "C" sssp_status sssp_mlp_backward(const float* w, const float* x, const f
   if (!w || !x || !target || !arm || !grad || batch == 0) return fail(SSSP_ERR_INVALID_ARG, "NULL or empty argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // one block per SM, and no more than the samples fill
-  const uint32_t tiles = (uint32_t)(((uint64_t)batch + kGradTile - 1) / kGradTile);
-  const int blocks = (int)std::min<uint32_t>(tiles, (uint32_t)sm_count());
+  const int blocks = (int)std::min<uint32_t>(grad_tiles(batch), (uint32_t)sm_count());
   TmpBuf<float> sbuf(st);
   sssp_status s = sbuf.alloc((size_t)blocks * kGradRow);
   if (s != SSSP_OK) return s;

@@ -1,0 +1,35 @@
+"""The training kernels at the ends of their ranges."""
+import numpy as np
+import pytest
+
+sp = pytest.importorskip("paper_1903_12085_gb300")
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _device():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("batch", [9, (1 << 32) - 7])
+def test_gradient_of_a_batch_as_large_as_its_count(batch):
+    """All samples alike, a network of zeros, every target 1: the loss is 1 and
+    the only gradient is -2, of the first output's bias.  Terms are powers of
+    two, at most 2^24 of them in a 32-bit sum, so what is left are the roundings
+    of batch (relative 2^-24, in 1/B) and of eight warps' sums: below 10 * 2^-24."""
+    if torch.cuda.mem_get_info()[0] < 41 * batch:
+        pytest.skip("not enough free device memory")
+    x = torch.zeros(batch, 8, device="cuda")
+    target = torch.ones(batch, device="cuda")
+    arm = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    grad, loss = sp.mlp_backward(torch.zeros(sp.POLICY_WEIGHTS, device="cuda"), x, target, arm)
+    grad = grad.cpu().numpy()
+    del x, target, arm
+    torch.cuda.empty_cache()
+    assert abs(float(loss.item()) - 1.0) <= 10 * 2.0 ** -24
+    assert abs(grad[-4] + 2.0) <= 20 * 2.0 ** -24
+    assert (np.delete(grad, -4 % grad.size) == 0).all()
