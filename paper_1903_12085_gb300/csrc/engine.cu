@@ -55,15 +55,16 @@ namespace sssp {
 #define SSSP_RARE(x) __builtin_expect(!!(x), 0)
 
 // What a kernel instance serves.  kAny: everything.  kArms: fused thresholds on
-// any of a policy's arms (IN-STATIC or IN-SIMPLE, sparse or dense), costs up to
-// kSoloNarrowW, nothing to record (trace, settle phases).  kStatic: the same on
-// static minima and the sparse queue alone.  They are kernels of their own: a
-// taken branch to code that is not in the instruction buffer costs 75 to 100
-// cycles (25 if it is; measured) and a phase takes dozens of them, and the
-// registers a step may use without saving them first depend on every other
-// function of its kernel.  (R-MAT s22 on the static criteria: 9.3 ms in an
-// instance that serves everything, 8.9 in its own.)
-enum { kAny = 0, kArms = 1, kStatic = 2 };
+// IN-STATIC or IN-SIMPLE, sparse or dense, costs up to kSoloNarrowW, nothing to
+// record (trace, settle phases).  kPolicy: the same with the choice left to a
+// policy.  kStatic: static minima and the sparse queue alone.  They are kernels
+// of their own: a taken branch to code that is not in the instruction buffer
+// costs 75 to 100 cycles (25 if it is; measured) and a phase takes dozens of
+// them, and the registers a step may use without saving them first depend on
+// every other function of its kernel.  (R-MAT s22 on the static criteria: 9.3 ms
+// in an instance that serves everything, 8.9 in its own.)
+enum { kAny = 0, kArms = 1, kStatic = 2, kPolicy = 3 };
+__host__ __device__ constexpr bool keeps_status(int kind) { return kind == kAny || kind == kArms; }
 
 // A group of co-resident blocks running one solve.  size == 1: block barriers.
 struct Grp {
@@ -122,16 +123,30 @@ __device__ __forceinline__ uint32_t out_min_dynamic(const GraphView& g, const So
   return cost;
 }
 
+// Whether v is in S, or in F: from the status bytes, or from the records in the
+// instance that keeps none (kPolicy).
+template <int kKind>
+__device__ __forceinline__ bool in_s(const SolveWS& w, uint32_t v) {
+  return kKind == kPolicy ? (ldcg_u64(&w.vrec[v].d) & kSettledBit) != 0 : ldcg_u8(&w.status[v]) == kS;
+}
+template <int kKind>
+__device__ __forceinline__ bool in_f(const SolveWS& w, uint32_t v) {
+  if (kKind != kPolicy) return ldcg_u8(&w.status[v]) == kF;
+  const unsigned long long d = ldcg_u64(&w.vrec[v].d);
+  return d != kUnexplored && !(d & kSettledBit);
+}
+
 // Advance the in-cursor of v past sources in S; return the dynamic in-minimum.
 // Concurrent callers for the same v compute the same position (S does not
 // change while they run), published with atomicMax.
+template <int kKind>
 __device__ __forceinline__ uint32_t in_min_dynamic(const GraphView& g, const SolveWS& w, uint32_t v, bool shared_v) {
   const uint32_t c0 = ldcg_u32(&w.cur_in[v]);
   const uint32_t end = (uint32_t)__ldg(&g.rrow_off[v + 1]);
   uint32_t c = c0, cost = kInf32;
   while (c < end) {
     const uint2 e = __ldg(&g.redges[c]);
-    if (ldcg_u8(&w.status[e.x]) != kS) { cost = e.y; break; }
+    if (!in_s<kKind>(w, e.x)) { cost = e.y; break; }
     ++c;
   }
   if (c != c0) {
@@ -253,7 +268,8 @@ struct Mode {
   // full/weak minima, APPROX and DIJK; with static criteria on the sparse queue
   // nothing reads them, so settling and discovering a vertex write none.  A
   // policy (its arms may scan densely or use IN-SIMPLE) needs them only until
-  // the fringe is split: from then on every phase runs its static sparse arm.
+  // the fringe is split: from then on every phase runs its static sparse arm;
+  // its own instance (kPolicy) never: there, the arms read the records.
   bool status;          // maintain the status bytes
   bool status_presplit;  // ... only while the fringe is not split
 };
@@ -519,7 +535,7 @@ __device__ __forceinline__ void relax_edge_rec(const SolveParams& p, const Mode&
     if (rt.d == kUnexplored) {
       old = atomicMin(&w.vrec[t].d, enc);
       if (old == kUnexplored) {
-        if (kKind != kStatic && status_live(md, kNF)) w.status[t] = kF;
+        if (keeps_status(kKind) && status_live(md, kNF)) w.status[t] = kF;
         if (kNF && (enc & kFarBit)) {
           ++dfar;
           if (nv.lists) app = nf_bucket(nv, enc, rt.im);
@@ -626,7 +642,7 @@ __device__ __noinline__ bool phase_select(bool alone, const Arm arm, uint64_t k,
   PhaseSlot* S0 = &ctl->slot[k % 4];
   PhaseSlot* S1 = &ctl->slot[(k + 1) % 4];
   const uint32_t nF = h.nQ;
-  const bool wstat = kKind != kStatic && status_live(md, h.split);
+  const bool wstat = keeps_status(kKind) && status_live(md, h.split);
   const bool dense = kKind != kStatic && arm.dense;
   const bool fused = kKind != kAny || md.fused, settle = kKind == kAny && w.settle_phase != nullptr;
   const bool in_dyn = kKind != kStatic && md.use_in && arm.in_simple && w.cur_in != nullptr;
@@ -649,11 +665,11 @@ __device__ __noinline__ bool phase_select(bool alone, const Arm arm, uint64_t k,
       // so advancing them lazily here is exact.
       if (dense) {
         for (uint64_t v = gtid; v < n; v += gthreads)
-          if (ldcg_u8(&w.status[v]) == kF) w.im_dyn[v] = in_min_dynamic(g, w, (uint32_t)v, false);
+          if (in_f<kKind>(w, (uint32_t)v)) w.im_dyn[v] = in_min_dynamic<kKind>(g, w, (uint32_t)v, false);
       } else {
         for (uint64_t i = gtid; i < nF; i += gthreads) {
           const uint32_t v = ldcg_u32(&Q[i]);
-          w.im_dyn[v] = in_min_dynamic(g, w, v, false);
+          w.im_dyn[v] = in_min_dynamic<kKind>(g, w, v, false);
         }
       }
       if (!grp.sync()) return false;
@@ -704,7 +720,7 @@ __device__ __noinline__ bool phase_select(bool alone, const Arm arm, uint64_t k,
         }
       }
       if (md.in_full) w.im_full[v] = in_min_full(g, w, v);
-      else if (in_dyn) w.im_dyn[v] = in_min_dynamic(g, w, v, false);
+      else if (in_dyn) w.im_dyn[v] = in_min_dynamic<kKind>(g, w, v, false);
       if (md.approx) {  // exact terms in every k-th phase, then APPROX's OUT threshold
         unsigned long long ao;
         if (apx_recompute) {
@@ -778,16 +794,16 @@ __device__ __noinline__ bool phase_select(bool alone, const Arm arm, uint64_t k,
     if (dense) {
 #pragma unroll
       for (int j = 0; j < kSelItems; ++j)
-        if (ok[j]) ok[j] = ldcg_u8(&w.status[vv[j]]) == kF;
+        if (ok[j] && kKind != kPolicy) ok[j] = ldcg_u8(&w.status[vv[j]]) == kF;
     }
     VRec rr[kSelItems];
 #pragma unroll
     for (int j = 0; j < kSelItems; ++j)
       if (ok[j]) rr[j] = ldcg_vrec(&w.vrec[vv[j]]);
-    if (dense && md.nearfar) {  // a dense scan also meets the far part of F
+    if (dense && (kKind == kPolicy || md.nearfar)) {  // a dense scan also meets the far part of F (and U and S: kUnexplored has the far bit set)
 #pragma unroll
       for (int j = 0; j < kSelItems; ++j)
-        if (ok[j] && (rr[j].d & kFarBit)) ok[j] = false;
+        if (ok[j] && (rr[j].d & (kKind == kPolicy ? kFarBit | kSettledBit : kFarBit))) ok[j] = false;
     }
     uint32_t selm = 0, keepm = 0;
     uint2 rd[kSelItems];
@@ -1187,7 +1203,7 @@ __device__ __noinline__ Arm policy_arm(uint64_t k, uint32_t nQ, uint32_t far) {
 
 template <int kKind>
 __device__ __forceinline__ bool run_phase(bool alone, uint64_t k, uint32_t nf_code, const PhaseHead& h) {
-  const bool policy = kKind != kStatic && (s_p.crit & SSSP_POLICY_LEARNED) && s_p.policy != nullptr;
+  const bool policy = kKind == kPolicy || (kKind == kAny && (s_p.crit & SSSP_POLICY_LEARNED) && s_p.policy != nullptr);
   const Arm arm = kKind == kStatic ? Arm{false, false, -1} : policy ? policy_arm(k, h.nQ, h.far) : arm_for(s_p, h.nQ);
   if (kKind == kAny) {
     const uint32_t size = alone ? 1u : s_grp.size, rank = alone ? 0u : s_grp.rank;
@@ -1378,6 +1394,103 @@ __device__ __noinline__ void solo_hand_off(uint32_t k, uint32_t live, uint32_t s
   }
 }
 
+// The arm of phase k of an episode, from the counters of the phase before; true
+// if its in-minima are the dynamic ones.
+template <bool kNF>
+__device__ __forceinline__ bool solo_choose(uint32_t k, bool first, uint32_t nF, uint32_t far) {
+  uint32_t e_prev, s_prev, f_prev;
+  if (first) {
+    const PhaseSlot* Sp = &s_p.ws.ctl->slot[(k + 3) % 4];
+    e_prev = (uint32_t)ldcg_u64(&Sp->relax_packed);
+    s_prev = ldcg_u32(&Sp->settled_now);
+    f_prev = ldcg_u32(&Sp->fsize);
+  } else {
+    const SoloCount* sp = &s_sc[(k + 1) & 1];
+    e_prev = sp->edges;
+    s_prev = sp->settled;
+    f_prev = nF + s_prev - sp->fresh + (kNF ? far - (uint32_t)sp->far : 0u);
+  }
+  const Arm arm = choose_arm(s_p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
+  if (threadIdx.x == 0) s_solo_arm = arm;  // (read past a barrier)
+  return arm.in_simple && s_md.use_in && s_p.ws.cur_in != nullptr;
+}
+
+// The in-minima that a phase compares with, of the live slots: the dynamic ones,
+// against the vertices settled before the phase (the barrier: before it marks
+// any), or the static ones again after such phases.  A warp's slots in use are
+// dealt to its lanes evenly: a cursor's round trips follow one another.
+template <class T, int kKind>
+__device__ __forceinline__ void solo_minima(uint32_t live, bool in_dyn) {
+  const SolveParams& p = s_p;
+  const SolveWS& w = p.ws;
+  const SoloMem<T> m = solo_carve<T>();
+  const unsigned int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
+  const uint32_t spt = p.solo_spt;
+  uint8_t* ids = reinterpret_cast<uint8_t*>(m.list);
+  static_assert(8 * 32 <= 256 && kSoloList * sizeof(uint4) >= 8 * 32, "eight slots a thread at a time");
+  for (uint32_t j0 = 0; j0 < spt; j0 += 8) {
+    uint32_t n = 0;
+    for (uint32_t j = 0; j < min(spt - j0, 8u); ++j) {
+      const bool on = (live >> (j0 + j)) & 1u;
+      const unsigned int bm = __ballot_sync(0xFFFFFFFFu, on);
+      if (on) ids[n + __popc(bm & ((1u << lane) - 1u))] = (uint8_t)(j * 32 + lane);
+      n += __popc(bm);
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < n; i += 32) {
+      const uint32_t s = (j0 + (ids[i] >> 5)) * nthr + warp * 32 + (ids[i] & 31u), v = m.slot[s].w;
+      m.slot[s].y = in_dyn ? in_min_dynamic<kKind>(p.g, w, v, false) : __ldg(&p.g.in_min[v]);
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+}
+
+// What an episode has to do about its arm, in one word: the low byte counts the
+// phases before the next choice, kEvDyn is set if the arm has dynamic in-minima
+// and kEvMinima if the slots' minima are to be computed in the next phase.  So a
+// phase has something to do only if the word is not positive.  (Without a policy
+// nothing is chosen again, and the count only starts over.)  One register, and
+// the work itself out of line: with the choice's phase, the arm and the work in
+// the episode's loop every phase paid for them (a policy that always keeps arm 0
+// on the 256 x 256 grid 12.7 ms, now 12.4; without a policy 11.5).
+constexpr uint32_t kEvMinima = 1u << 31, kEvDyn = 1u << 30;
+__device__ __forceinline__ bool solo_policy() { return (s_p.crit & SSSP_POLICY_LEARNED) != 0; }
+
+template <bool kNF>
+__device__ __forceinline__ uint32_t solo_begin(uint32_t k, uint32_t nF, uint32_t far) {
+  bool dyn;
+  uint32_t count = solo_policy() ? 8u : 0xFFu;
+  if (s_solo_cont && (!solo_policy() || s_solo_since)) {
+    if (solo_policy()) count -= s_solo_since;
+    dyn = s_solo_arm.in_simple && s_md.use_in && s_p.ws.cur_in != nullptr;
+  } else {
+    dyn = solo_choose<kNF>(k, true, nF, far);
+  }
+  return count | (dyn ? kEvMinima | kEvDyn : 0u);
+}
+
+template <class T, bool kNF, int kKind>
+__device__ __forceinline__ uint32_t solo_event(uint32_t ev, uint32_t k, uint32_t nF, uint32_t far, uint32_t live) {
+  if ((ev & 0xFFu) == 0) {
+    if (!solo_policy()) ev |= 0xFFu;
+    else ev = (ev & kEvMinima) | 8u | (solo_choose<kNF>(k, false, nF, far) ? kEvDyn : 0u);
+  }
+  if (ev & (kEvMinima | kEvDyn)) solo_minima<T, kKind>(live, (ev & kEvDyn) != 0);
+  return (ev & kEvDyn) ? ev | kEvMinima : ev & ~kEvMinima;
+}
+
+// (inlined in the general instance: calls would take registers from its steps,
+// 8 sources of G(2^24, 2^28) at once 116.9 -> 117.6 ms)
+template <bool kNF>
+__device__ __noinline__ uint32_t solo_begin_call(uint32_t k, uint32_t nF, uint32_t far) {
+  return solo_begin<kNF>(k, nF, far);
+}
+template <class T, bool kNF, int kKind>
+__device__ __noinline__ uint32_t solo_event_call(uint32_t ev, uint32_t k, uint32_t nF, uint32_t far, uint32_t live) {
+  return solo_event<T, kNF, kKind>(ev, k, nF, far, live);
+}
+
 // T = uint32_t: D is rebased once minD has moved this far from the base, and a
 // vertex settled with a D past the second limit (which static criteria never
 // reach: a fringe lies within twice the largest cost of its minD) ends the
@@ -1405,9 +1518,8 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
   const bool scribe = tid == nthr - 32;  // writes the trace, waits for the group
   const uint32_t spt = p.solo_spt;       // slots per thread (at most 16)
   const bool use_in = s_md.use_in, use_out = s_md.use_out;
-  uint8_t* const status = kKind != kStatic && status_live(s_md, kNF) ? w.status : nullptr;
+  uint8_t* const status = keeps_status(kKind) && status_live(s_md, kNF) ? w.status : nullptr;
   const bool settle = kKind == kAny && w.settle_phase != nullptr, trace = kKind == kAny && w.trace != nullptr;
-  const bool policy = kKind != kStatic && (p.crit & SSSP_POLICY_LEARNED) != 0;
   const SoloMem<T> m = solo_carve<T>();
   __shared__ unsigned long long s_t0, s_tsel;  // trace stamps
   __shared__ uint2 s_warp[32];  // per warp: edges of the phase, settled vertices
@@ -1424,16 +1536,10 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     minD = (T)(d - base);
     minOut = o - base > inf ? inf : (T)(o - base);
   }
-  // The arm (s_solo_arm) is chosen in phase `pick`: the policy's in the first phase
-  // of the episode and every 8th after it (the choice is logged per phase either way).
-  uint32_t pick = k;
-  bool in_dyn = false;
-  if (kKind != kStatic && s_solo_cont) {
-    const uint32_t since = s_solo_since;
-    pick = !policy ? kInf32 : since ? k + 8 - since : k;
-    in_dyn = s_solo_arm.in_simple && use_in && w.cur_in != nullptr;
-  }
-  const uint32_t k_first = k;
+  // The arm (s_solo_arm) is chosen in the first phase of the episode and, with a
+  // policy, every 8th after it (the choice is logged per phase either way).
+  uint32_t ev = 0;
+  if (kKind != kStatic) ev = kKind == kAny ? solo_begin<kNF>(k, nF, far) : solo_begin_call<kNF>(k, nF, far);
   // counters of the episode
   unsigned long long sum_f = 0, sum_s = 0, sum_e = 0;
   if (tid == 0) solo_clear(&s_sc[k & 1]);
@@ -1466,53 +1572,15 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
   if (tid == 0) s_solo_cont = 0;
   T od, oo;
   uint32_t sel;
-  bool hand = false, was_dyn = false;
+  bool hand = false;
 
   for (;;) {
     SoloCount* const sc = &s_sc[k & 1];
-    if (kKind != kStatic && SSSP_RARE(k == pick)) {
-      uint32_t e_prev, s_prev, f_prev;  // counters of the last phase
-      if (k == k_first) {
-        const PhaseSlot* Sp = &ctl->slot[(k + 3) % 4];
-        e_prev = (uint32_t)ldcg_u64(&Sp->relax_packed);
-        s_prev = ldcg_u32(&Sp->settled_now);
-        f_prev = ldcg_u32(&Sp->fsize);
-      } else {
-        const SoloCount* sp = &s_sc[(k + 1) & 1];
-        e_prev = sp->edges;
-        s_prev = sp->settled;
-        f_prev = nF + s_prev - sp->fresh + (kNF ? far - (uint32_t)sp->far : 0u);
-      }
-      const Arm arm = choose_arm(p, k, nF, nF + far, e_prev, s_prev, f_prev, kNF);
-      if (tid == 0) s_solo_arm = arm;  // (read past a barrier)
-      pick = policy ? k + 8 : kInf32;
-      in_dyn = arm.in_simple && use_in && w.cur_in != nullptr;
-    }
     if (scribe && trace) s_t0 = globaltimer_ns();
     live = m.used[tid] & ~spent;
-    if (kKind != kStatic && SSSP_RARE(in_dyn || was_dyn)) {  // minima of this phase's variant (IN-SIMPLE reads status bytes the selection writes)
-      // (the warp's slots in use, dealt to its lanes evenly: a cursor's round
-      // trips follow one another)
-      uint8_t* ids = reinterpret_cast<uint8_t*>(m.list);
-      static_assert(8 * 32 <= 256 && kSoloList * sizeof(uint4) >= 8 * 32, "eight slots a thread at a time");
-      for (uint32_t j0 = 0; j0 < spt; j0 += 8) {
-        uint32_t n = 0;
-        for (uint32_t j = 0; j < min(spt - j0, 8u); ++j) {
-          const bool on = (live >> (j0 + j)) & 1u;
-          const unsigned int bm = __ballot_sync(0xFFFFFFFFu, on);
-          if (on) ids[n + __popc(bm & ((1u << lane) - 1u))] = (uint8_t)(j * 32 + lane);
-          n += __popc(bm);
-        }
-        __syncwarp();
-        for (uint32_t i = lane; i < n; i += 32) {
-          const uint32_t s = (j0 + (ids[i] >> 5)) * nthr + warp * 32 + (ids[i] & 31u), v = m.slot[s].w;
-          m.slot[s].y = in_dyn ? in_min_dynamic(p.g, w, v, false) : __ldg(&p.g.in_min[v]);
-        }
-        __syncwarp();
-      }
-      was_dyn = in_dyn;
-      __syncthreads();
-    }
+    if (kKind != kStatic && SSSP_RARE((int)ev <= 0))
+      ev = kKind == kAny ? solo_event<T, kNF, kKind>(ev, k, nF, far, live)
+                         : solo_event_call<T, kNF, kKind>(ev, k, nF, far, live);
     if (kNarrow && SSSP_RARE(minD > kSoloRebase)) {
       for (uint32_t b = live; b; b &= b - 1) *m.d((uint32_t)(__ffs(b) - 1) * nthr + tid) -= minD;
       base += minD;
@@ -1562,7 +1630,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
           if (at < kSoloList)
             m.list[at] = make_uint4(row.x, row.y, (uint32_t)dv, (uint32_t)((unsigned long long)dv >> 32));
           vrec[v].d = (base + dv) | kSettledBit;
-          if (kKind != kStatic && status) status[v] = kS;
+          if (keeps_status(kKind) && status) status[v] = kS;
           if (settle) w.settle_phase[v] = k;
           if (kNarrow && dv > kSoloLastD) sc->stop = 1;
         }
@@ -1696,7 +1764,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
           om = mm.y;
           claimed = x == kUnexplored;
           lowered = !(x & kSettledBit);
-          if (kKind != kStatic && claimed && status) status[t] = kF;
+          if (keeps_status(kKind) && claimed && status) status[t] = kF;
           x = claimed ? s : x;
         } else {
           const VRec r = ldcg_vrec(&vrec[t]);
@@ -1714,7 +1782,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
               lowered = enc < x;
               if (x == kUnexplored) {
                 ++nfar;
-                if (kKind != kStatic && status) status[t] = kF;
+                if (keeps_status(kKind) && status) status[t] = kF;
                 if (nv.lists) app = nf_bucket(nv, enc, im);
               } else if (lowered && nv.lists) {
                 const uint32_t b = nf_bucket(nv, enc, im);
@@ -1728,7 +1796,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
               if (o == x) {
                 claimed = true;
                 if (x != kUnexplored) --nfar;
-                else if (kKind != kStatic && status) status[t] = kF;
+                else if (keeps_status(kKind) && status) status[t] = kF;
                 trow = __ldg(&rowdeg[t]);
                 x = s;
               } else {
@@ -1786,7 +1854,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
       r.min_out = use_out && minOut != inf ? base + minOut : kInf64;
       r.deg_settled = E;
       uint32_t c = p.crit & SSSP_CRITERIA_MASK;
-      if (use_in) c = (c & ~(uint32_t)(SSSP_IN_STATIC | SSSP_IN_SIMPLE)) | (in_dyn ? SSSP_IN_SIMPLE : SSSP_IN_STATIC);
+      if (use_in) c = (c & ~(uint32_t)(SSSP_IN_STATIC | SSSP_IN_SIMPLE)) | ((ev & kEvDyn) ? SSSP_IN_SIMPLE : SSSP_IN_STATIC);
       r.criterion = c;
       r.arm = arm_code(s_solo_arm, true) | nf_code;
       r.t_start_ns = s_t0;
@@ -1801,6 +1869,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     minD = *solo_thr<T>(&sc->min_d);
     minOut = use_out ? *solo_thr<T>(&sc->min_out) : inf;
     ++k;
+    --ev;
     if (nF == 0 || nF > solo_stay(p) || k > p.g.n + 1) break;
     // thresholds above the bound are exact only after the far part is scanned
     if (kNF && far > 0) {
@@ -1819,7 +1888,7 @@ __device__ __noinline__ uint64_t solo_episode(uint32_t k, uint32_t nf_code, bool
     solo_hand_off<T>(k, live & ~sel, sel, od, oo, base, minD, minOut, nF, far, nf_code, s_t0);
     if (tid == 0 && (!group || (uint32_t)s_solo_n <= p.solo_edges)) {
       s_solo_cont = 1;
-      s_solo_since = policy ? (k + 9 - pick) & 7u : 1u;
+      s_solo_since = kKind != kStatic && solo_policy() ? (9 - (ev & 0xFFu)) & 7u : 1u;
     }
     __threadfence();
     __syncthreads();
@@ -2680,14 +2749,16 @@ int kind_of(uint32_t crit, bool narrow, bool records) {
   constexpr uint32_t is = SSSP_IN_STATIC | SSSP_OUT_STATIC;
   constexpr uint32_t arms = is | SSSP_IN_SIMPLE | SSSP_POLICY_LEARNED | SSSP_FRONTIER_DENSE | SSSP_FRONTIER_AUTO;
   if (!narrow || records || (crit & ~arms)) return kAny;
-  return (crit & ~is) ? kArms : kStatic;
+  return (crit & SSSP_POLICY_LEARNED) ? kPolicy : (crit & ~is) ? kArms : kStatic;
 }
 int solve_kind(const SolveParams& p) {
   return kind_of(p.crit, p.g.max_w <= kSoloNarrowW, p.ws.trace || p.ws.settle_phase || !p.ws.tile_owner);
 }
 const void* grid_kernel(int kind) {
-  return kind == kStatic ? (const void*)k_solve_grid<kStatic>
-                         : kind == kArms ? (const void*)k_solve_grid<kArms> : (const void*)k_solve_grid<kAny>;
+  return kind == kStatic   ? (const void*)k_solve_grid<kStatic>
+         : kind == kPolicy ? (const void*)k_solve_grid<kPolicy>
+         : kind == kArms   ? (const void*)k_solve_grid<kArms>
+                           : (const void*)k_solve_grid<kAny>;
 }
 
 namespace {
@@ -2711,8 +2782,10 @@ int current_device() {
 
 template <int kT>
 const void* batch_kernel_of(int kind) {
-  return kind == kStatic ? (const void*)k_solve_batch<kStatic, kT>
-                         : kind == kArms ? (const void*)k_solve_batch<kArms, kT> : (const void*)k_solve_batch<kAny, kT>;
+  return kind == kStatic   ? (const void*)k_solve_batch<kStatic, kT>
+         : kind == kPolicy ? (const void*)k_solve_batch<kPolicy, kT>
+         : kind == kArms   ? (const void*)k_solve_batch<kArms, kT>
+                           : (const void*)k_solve_batch<kAny, kT>;
 }
 const void* batch_kernel(int kind, uint32_t threads) {
   return threads == kThreads ? batch_kernel_of<kThreads>(kind) : batch_kernel_of<kSmallThreads>(kind);
@@ -2725,7 +2798,7 @@ sssp_status ensure_kernel_attrs() {
   std::lock_guard<std::mutex> lock(g_attr_mu);
   if (g_blocks_per_sm[dev].load() > 0) return SSSP_OK;
   int per_sm = 1 << 10;
-  for (int kind : {kAny, kArms, kStatic}) {
+  for (int kind : {kAny, kArms, kStatic, kPolicy}) {
     for (const void* kernel : {grid_kernel(kind), batch_kernel(kind, kThreads), batch_kernel(kind, kSmallThreads)}) {
       const bool small = kernel == batch_kernel(kind, kSmallThreads);
       const int threads = small ? kSmallThreads : kThreads;
@@ -2969,8 +3042,8 @@ struct BatchPlan {
   uint32_t recording = 0;              // solves with a trace or settle phases attached
   // Policy solves of graphs with small episodes (solo_large) run mostly grid
   // phases, whose steps spill least in the batch's general instance: 8 sources of
-  // G(2^24, 2^28) at once 119 ms, in the instance for the arms 121.4.  (Single
-  // solves are the other way round: G(2^20, 2^24) 8.6 and 8.2 ms.)
+  // G(2^24, 2^28) at once 117 ms, in the policy's own 122.  (Single solves are
+  // the other way round: G(2^20, 2^24) 8.6 and 8.0 ms.)
   int kind() const { return kind_of(crit, narrow, recording != 0 || (!large && (crit & SSSP_POLICY_LEARNED))); }
   uint32_t bpg = 1;                    // blocks per solve
   bool staged = false;                 // bpg = 1: larger solves get more blocks
