@@ -108,14 +108,14 @@ k_mlp_grad(const float* __restrict__ w, const float* __restrict__ x, const float
       my_a = my_a < (uint32_t)kPolArms ? my_a : 0u;
     }
     __syncwarp();
-    for (int s = 0; s < n; s += 2) {  // (an odd last sample's twin counts for nothing: its error is zeroed)
+    for (int s = 0; s < n; s += 2) {  // (an odd last sample's twin counts for nothing: its activations and error are zero)
       float h1[2], h2[2], g[2];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         float z = b1;
 #pragma unroll
         for (int i = 0; i < kPolFeat; ++i) z = fmaf(s_x[warp][s + u][i], w1[i], z);
-        h1[u] = fmaxf(z, 0.0f);
+        h1[u] = s + u < n ? fmaxf(z, 0.0f) : 0.0f;
         s_h[warp][u][lane] = h1[u];
       }
       __syncwarp();
@@ -124,7 +124,7 @@ k_mlp_grad(const float* __restrict__ w, const float* __restrict__ x, const float
         float z = b2;
 #pragma unroll
         for (int i = 0; i < kPolHidden; ++i) z = fmaf(s_h[warp][u][i], w2c[i], z);
-        h2[u] = fmaxf(z, 0.0f);
+        h2[u] = s + u < n ? fmaxf(z, 0.0f) : 0.0f;
       }
       float ya[2];
       uint32_t a[2];

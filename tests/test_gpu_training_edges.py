@@ -33,3 +33,21 @@ def test_gradient_of_a_batch_as_large_as_its_count(batch):
     assert abs(float(loss.item()) - 1.0) <= 10 * 2.0 ** -24
     assert abs(grad[-4] + 2.0) <= 20 * 2.0 ** -24
     assert (np.delete(grad, -4 % grad.size) == 0).all()
+
+
+@pytest.mark.parametrize("batch", [1, 9])
+def test_an_odd_sample_is_alone(batch):
+    """A first layer that is zero on every sample and overflows the second where
+    there is none: all activations are zero, so the only gradient is the first
+    output bias's, 2 (0 - 1), exactly up to the roundings of 1/B and the sums."""
+    w = torch.zeros(sp.POLICY_WEIGHTS, device="cuda")
+    w[0], w[256] = -2e38, 2e38  # W1[0][0], b1[0]
+    w[288] = 2.0  # W2[0][0]
+    x = torch.zeros(batch, 8, device="cuda")
+    x[:, 0] = 1.0
+    arm = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    grad, loss = sp.mlp_backward(w, x, torch.ones(batch, device="cuda"), arm)
+    grad = grad.cpu().numpy()
+    assert abs(float(loss.item()) - 1.0) <= 10 * 2.0 ** -24
+    assert abs(grad[-4] + 2.0) <= 20 * 2.0 ** -24
+    assert (np.delete(grad, -4 % grad.size) == 0).all()
