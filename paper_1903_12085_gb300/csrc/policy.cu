@@ -31,7 +31,8 @@ __global__ void k_mlp_forward(const float* __restrict__ w, const float* __restri
   __shared__ float sw[kPolWeights];
   for (int i = threadIdx.x; i < kPolWeights; i += blockDim.x) sw[i] = w[i];
   __syncthreads();
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x) {
+  // (64 bits: near 2^32 samples a 32-bit counter would wrap and never end)
+  for (uint64_t b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x) {
     float h1[kPolHidden], h2[kPolHidden];
     for (int j = 0; j < kPolHidden; ++j) {
       float z = sw[kPolOffB1 + j];
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256) k_mlp_grad_reduce(const float* __restrict
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m1,
                        float* __restrict__ m2, uint32_t count, float lr, float beta1, float beta2, float eps,
                        float c1, float c2) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float a = beta1 * m1[i] + (1.0f - beta1) * gi;
     const float b = beta2 * m2[i] + (1.0f - beta2) * gi * gi;
@@ -286,7 +287,7 @@ extern "C" sssp_status sssp_mlp_forward(const float* w, const float* x, uint32_t
   if (!w || !x || !y) return fail(SSSP_ERR_INVALID_ARG, "NULL argument");
   if (batch == 0) return SSSP_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int blocks = (int)std::min<uint32_t>((batch + 127) / 128, 1024);
+  const int blocks = (int)std::min<uint64_t>(((uint64_t)batch + 127) / 128, 1024);
   k_mlp_forward<<<blocks, 128, 0, st>>>(w, x, batch, y);
   SSSP_CUDA_TRY(cudaGetLastError());
   return SSSP_OK;
@@ -313,7 +314,7 @@ extern "C" sssp_status sssp_mlp_adam(float* w, const float* grad, float* m1, flo
   clear_error();
   if (!w || !grad || !m1 || !m2 || step == 0) return fail(SSSP_ERR_INVALID_ARG, "bad Adam arguments");
   const float c1 = 1.0f - powf(beta1, (float)step), c2 = 1.0f - powf(beta2, (float)step);
-  k_adam<<<(int)std::min<uint32_t>((count + 255) / 256, 1024), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+  k_adam<<<(int)std::min<uint64_t>(((uint64_t)count + 255) / 256, 1024), 256, 0, static_cast<cudaStream_t>(stream)>>>(
       w, grad, m1, m2, count, lr, beta1, beta2, eps, c1, c2);
   SSSP_CUDA_TRY(cudaGetLastError());
   return SSSP_OK;

@@ -51,3 +51,33 @@ def test_an_odd_sample_is_alone(batch):
     assert abs(float(loss.item()) - 1.0) <= 10 * 2.0 ** -24
     assert abs(grad[-4] + 2.0) <= 20 * 2.0 ** -24
     assert (np.delete(grad, -4 % grad.size) == 0).all()
+
+
+@pytest.mark.parametrize("count", [129, (1 << 32) - 7])
+def test_forward_of_a_batch_as_large_as_its_count(count):
+    """Outputs of the first and last samples: the output biases, exactly."""
+    if torch.cuda.mem_get_info()[0] < 49 * count:
+        pytest.skip("not enough free device memory")
+    w = torch.zeros(sp.POLICY_WEIGHTS, device="cuda")
+    w[-4:] = torch.arange(1.0, 5.0)
+    y = sp.mlp_forward(w, torch.zeros(count, 8, device="cuda"))
+    ends = torch.cat([y[:3], y[-3:]]).cpu()
+    del y
+    torch.cuda.empty_cache()
+    assert (ends == torch.arange(1.0, 5.0)).all()
+
+
+@pytest.mark.parametrize("count", [257, (1 << 32) - 7])
+def test_adam_of_as_many_weights_as_its_count(count):
+    """A first step from zero moments moves every weight by the rate (both bias
+    corrections cancel the decay factors, eps is 0), up to the roundings of
+    about eight operations."""
+    if torch.cuda.mem_get_info()[0] < 17 * count:
+        pytest.skip("not enough free device memory")
+    w, m1, m2 = (torch.zeros(count, device="cuda") for _ in range(3))
+    grad = torch.ones(count, device="cuda")
+    sp.mlp_adam(w, grad, m1, m2, lr=0.5, step=1, eps=0.0)
+    ends = torch.cat([w[:3], w[-3:]]).cpu()
+    del w, m1, m2, grad
+    torch.cuda.empty_cache()
+    assert ((ends + 0.5).abs() <= 0.5 * 2.0 ** -20).all()
