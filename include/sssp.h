@@ -221,7 +221,9 @@ sssp_status sssp_solve_batch(sssp_graph* const* graphs, const uint32_t* sources,
  * at creation.  phases_out must be device memory here.  With
  * SSSP_POLICY_LEARNED the batch copies the policy network loaded at creation
  * and uses that copy in every launch (loading or clearing a network later does
- * not affect it); its graphs need SSSP_GRAPH_REVERSE for the IN-SIMPLE arms. */
+ * not affect it); its graphs need SSSP_GRAPH_REVERSE for the IN-SIMPLE arms.
+ * Tuning and wait limit are those of its creation, or of its last
+ * sssp_batch_autotune, in every launch. */
 typedef struct sssp_batch sssp_batch;
 sssp_status sssp_batch_create(sssp_graph* const* graphs, const uint32_t* sources, uint32_t count,
                               uint32_t criterion, uint64_t* const* dist_out, uint64_t* phases_out,
@@ -234,7 +236,9 @@ void sssp_batch_destroy(sssp_batch* b);
  * phase in which each vertex settled (0 = never) to `settle_phase`, both
  * device memory owned by the caller (NULL stops that output).  The records are
  * those of sssp_solve_trace; with SSSP_POLICY_LEARNED they give the arm each
- * phase ran with, so the schedule of a batched solve can be replayed.  Call it
+ * phase ran with, so the schedule of a batched solve can be replayed.  The first
+ * solve that records, and the end of the last, capture the launch anew (another
+ * kernel instance, the same tuning); if that fails the batch stays as it was.  Call it
  * when no launch of the batch is in flight; synchronous on `stream`.  A
  * library feature with no counterpart in the paper. */
 sssp_status sssp_batch_trace(sssp_batch* b, uint32_t i, sssp_phase_record* trace, uint64_t trace_cap,

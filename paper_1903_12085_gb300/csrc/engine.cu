@@ -3045,6 +3045,8 @@ struct BatchPlan {
   // G(2^24, 2^28) at once 117 ms, in the policy's own 122.  (Single solves are
   // the other way round: G(2^20, 2^24) 8.6 and 8.0 ms.)
   int kind() const { return kind_of(crit, narrow, recording != 0 || (!large && (crit & SSSP_POLICY_LEARNED))); }
+  BatchTuning tuning{};                // in force when the batch was created (or autotuned last)
+  unsigned long long wait_ns = 0;      // the wait limit then
   uint32_t bpg = 1;                    // blocks per solve
   bool staged = false;                 // bpg = 1: larger solves get more blocks
   uint32_t slots = 0;                  // gslots allocated (any stages fit)
@@ -3142,6 +3144,12 @@ LaunchPlan batch_plan(const BatchPlan& b) {
   return l;
 }
 
+// The batch's launches use the tuning and the wait limit of this moment.
+void batch_take_tuning(sssp_batch* b) {
+  b->tuning = BatchTuning{solo_max(), solo_edges(), nearfar_min(), nearfar_target(), nearfar_share(), 0, 0};
+  b->wait_ns = wait_limit_ns();
+}
+
 // Queue the batch on `st`: reset the work counter, group slots and every
 // control block, then one cooperative launch whose groups pull solves.
 sssp_status batch_enqueue(sssp_batch* b, cudaStream_t st) {
@@ -3150,10 +3158,9 @@ sssp_status batch_enqueue(sssp_batch* b, cudaStream_t st) {
   SSSP_CUDA_TRY(cudaMemsetAsync(b->gslots, 0, b->slots * sizeof(GroupSlot), st));
   SSSP_CUDA_TRY(cudaMemsetAsync(b->err, 0, sizeof(int), st));
   for (Workspace* w : b->ws) SSSP_CUDA_TRY(cudaMemsetAsync(w->ctl, 0, sizeof(Ctl), st));
-  BatchTuning tu{solo_max(), solo_edges(), nearfar_min(), nearfar_target(), nearfar_share(), 0, 0};
+  BatchTuning tu = b->tuning;
   const size_t smem = solo_shape_of(l.threads == kThreads ? b->large : b->mesh, b->narrow, b->crit, l.threads, &tu);
-  unsigned long long wait = wait_limit_ns();
-  void* args[] = {&b->items, &b->next, &b->gslots, &l.stages, &b->crit, &tu, &wait, &b->err, &b->phases, &b->policy};
+  void* args[] = {&b->items, &b->next, &b->gslots, &l.stages, &b->crit, &tu, &b->wait_ns, &b->err, &b->phases, &b->policy};
   SSSP_CUDA_TRY(cudaLaunchCooperativeKernel(batch_kernel(b->kind(), l.threads), dim3(l.blocks), dim3(l.threads), args,
                                             smem, st));
   return SSSP_OK;
@@ -3197,6 +3204,7 @@ sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint
   }
   b->bpg = bpg;
   b->staged = !tuned && bpg == 1;
+  batch_take_tuning(b);
   b->slots = kMaxStages * resident * (kThreads / kSmallThreads);
   // Largest solves first, so the tail of the queue holds the short ones.
   std::vector<uint32_t> order(count);
@@ -3255,31 +3263,32 @@ sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint
   return SSSP_OK;
 }
 
-// Capture the batch's launch (current blocks per solve) in a CUDA graph.
+// Capture the batch's launch (current blocks per solve and kernel instance) in a
+// CUDA graph, in place of the one it has (no launch of the batch is in flight).
+// On failure the batch keeps the graph it had.
 sssp_status batch_capture(sssp_batch* b) {
   cudaStream_t cap = nullptr;
   if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess)
     return fail(SSSP_ERR_CUDA, "stream creation failed");
   sssp_status s = SSSP_OK;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     s = batch_enqueue(b, cap);
-    e = cudaStreamEndCapture(cap, &b->graph);
+    e = cudaStreamEndCapture(cap, &graph);
   }
-  if (e == cudaSuccess && s == SSSP_OK) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+  if (e == cudaSuccess && s == SSSP_OK) e = cudaGraphInstantiate(&exec, graph, 0);
   cudaStreamDestroy(cap);
-  if (s != SSSP_OK) return s;
-  if (e != cudaSuccess) return fail(SSSP_ERR_CUDA, "CUDA graph capture failed: %s", cudaGetErrorString(e));
-  return SSSP_OK;
-}
-
-// Capture it anew (no launch of the batch is in flight).
-sssp_status batch_recapture(sssp_batch* b) {
+  if (s != SSSP_OK || e != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
+    return s != SSSP_OK ? s : fail(SSSP_ERR_CUDA, "CUDA graph capture failed: %s", cudaGetErrorString(e));
+  }
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
-  b->exec = nullptr;
-  b->graph = nullptr;
-  return batch_capture(b);
+  b->exec = exec;
+  b->graph = graph;
+  return SSSP_OK;
 }
 
 sssp_status batch_status(sssp_batch* b) {
@@ -3360,6 +3369,7 @@ extern "C" sssp_status sssp_batch_autotune(sssp_batch* b, void* stream, uint32_t
   if (!b) return fail(SSSP_ERR_INVALID_ARG, "batch is NULL");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const uint32_t resident = resident_blocks();
+  batch_take_tuning(b);
   // candidates: 1, 2, 4, ..., all co-resident blocks, and the batch's own
   // choice.  The search starts at the batch's choice and walks up and then
   // down the ladder; a walk stops at the first candidate that is clearly
@@ -3430,7 +3440,7 @@ extern "C" sssp_status sssp_batch_autotune(sssp_batch* b, void* stream, uint32_t
   for (auto& e : ev) cudaEventDestroy(e);
   b->bpg = s == SSSP_OK ? best : bpg0;
   b->staged = own && b->bpg == bpg0;
-  const sssp_status sc = batch_recapture(b);
+  const sssp_status sc = batch_capture(b);
   if (s != SSSP_OK) return s;
   if (sc != SSSP_OK) return sc;
   if (bpg_out) *bpg_out = best;
@@ -3448,17 +3458,28 @@ extern "C" sssp_status sssp_batch_trace(sssp_batch* b, uint32_t i, sssp_phase_re
   uint32_t k = 0;
   while (k < b->count && b->h_items[k].out_index != i) ++k;
   if (k == b->count) return fail(SSSP_ERR_INTERNAL, "solve %u has no descriptor", i);
-  BatchItem& it = b->h_items[k];
-  const bool was = it.ws.trace || it.ws.settle_phase;
+  BatchItem it = b->h_items[k];
+  const uint32_t recording = b->recording;
   const int kind = b->kind();
+  const bool was = it.ws.trace || it.ws.settle_phase;
   it.ws.trace = trace_cap ? trace : nullptr;
   it.ws.trace_cap = trace ? trace_cap : 0;
   it.ws.settle_phase = settle_phase;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   b->recording += (it.ws.trace || it.ws.settle_phase ? 1u : 0u) - (was ? 1u : 0u);
+  // The records need the general instance: a first one (and the end of the last)
+  // has the launch captured anew, with the tuning it had.
+  if (b->kind() != kind) {
+    const sssp_status s = batch_capture(b);
+    if (s != SSSP_OK) {
+      b->recording = recording;
+      return s;
+    }
+  }
+  b->h_items[k] = it;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
   SSSP_CUDA_TRY(cudaMemcpyAsync(&b->items[k], &it, sizeof(BatchItem), cudaMemcpyHostToDevice, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));
-  return b->kind() == kind ? SSSP_OK : batch_recapture(b);  // (the other kernel from now on)
+  return SSSP_OK;
 }
 
 extern "C" sssp_status sssp_batch_launch(sssp_batch* b, void* stream) {
