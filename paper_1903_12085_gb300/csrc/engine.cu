@@ -337,6 +337,9 @@ __device__ __forceinline__ uint32_t solo_limit(const SolveParams& p, uint32_t ei
   const bool policy = (p.crit & SSSP_POLICY_LEARNED) != 0;
   return p.solo_max < kSoloCap || policy ? min(p.solo_max, kSoloCap) : p.solo_spt * blockDim.x / 8 * eighths;
 }
+// The phases of the three-step kind on one block keep the fringe in global
+// memory, so no slots speak for more than kSoloCap.
+__device__ __forceinline__ uint32_t generic_limit(const SolveParams& p) { return min(p.solo_max, kSoloCap); }
 __device__ __forceinline__ uint32_t solo_enter(const SolveParams& p) { return solo_limit(p, 5); }
 __device__ __forceinline__ uint32_t solo_stay(const SolveParams& p) { return solo_limit(p, 6); }
 
@@ -2482,7 +2485,7 @@ __device__ __noinline__ uint64_t generic_solo(uint64_t k) {
   // (ordered by the barriers of phase k; the queue length, all that the others
   // read of the head for these criteria, is reset in phase k + 2)
   if (threadIdx.x == blockDim.x - 32) episode_join();
-  while (h.nQ != 0 && h.nQ <= p.solo_max && k <= (uint64_t)p.g.n + 1) {
+  while (h.nQ != 0 && h.nQ <= generic_limit(p) && k <= (uint64_t)p.g.n + 1) {
     run_phase<kAny>(true, k, 0u, h);
     ++k;
     if (threadIdx.x == 0) ctl->heartbeat = k;
@@ -2599,7 +2602,7 @@ __device__ __forceinline__ void solve_body(const Grp& grp_in) {
     // policy's phases keep to the fringe's size)
     const bool fast_solo = md.fused && (p.crit & SSSP_FRONTIER_DENSE) == 0 && h.nQ <= solo_enter(p) &&
                            (h.e_prev <= p.solo_edges || grp.size == 1 || (p.crit & SSSP_POLICY_LEARNED));
-    const bool three_step_solo = kKind == kAny && !md.fused && grp.size > 1 && h.nQ <= p.solo_max;
+    const bool three_step_solo = kKind == kAny && !md.fused && grp.size > 1 && h.nQ <= generic_limit(p);
     if ((fast_solo || three_step_solo) && !forced) {
       uint64_t r;  // 4 k + kSoloResume or kSoloNoFit
       if (grp.rank == 0) {
