@@ -347,8 +347,9 @@ sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t* row_offse
  * the block has room for beside the phase's new vertices, some 1300 to 3000; with
  * SSSP_POLICY_LEARNED 2048; for criteria other than IN-STATIC, IN-SIMPLE and
  * OUT-STATIC at most 2048, with the fringe in global memory); if its relax list
- * then has more than solo_max_edges edges, the relax step is handed to all blocks
- * of the solve (not for those other criteria);
+ * then has more than solo_max_edges edges (half as many again if the phase before
+ * ran so too, and without SSSP_POLICY_LEARNED), the relax step is handed to all
+ * blocks of the solve (not for those other criteria);
  * batch_blocks_per_solve: blocks that cooperate on one solve of a batch (0 =
  * chosen from the batch); grid_blocks: blocks of a single solve (0 = chosen
  * from n, capped at the co-resident maximum);

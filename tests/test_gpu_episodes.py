@@ -44,3 +44,24 @@ def test_groups_and_their_leader_agree(crit, ends):
             outs, phases = sp.solve_batch([G] * 12, [1] * 12, crit)
             assert all((sp.as_uint64(o) == ref).all() for o in outs) and (phases == sim.phases).all(), (g.name, blocks)
         G.close()
+
+
+@pytest.mark.parametrize("edges", [0, 1, 7, 2048, 0xFFFFFFFF])
+def test_edge_limits_of_an_episode(edges):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    try:
+        for g in (gg.rmat(11, 19, 0.57, 0.19, 0.19, 0, 1 << 24, 64), gg.gnm(900, 30000, 0, 1 << 24, 65)):
+            G = sp.Graph.from_csr(g)
+            ref = oracle.dijkstra(g, 1)
+            sim = oracle.simulate(g, 1, sp.IN_OUT, dist_ref=ref)
+            for blocks in (1, 3):
+                sp.set_tuning()
+                sp.set_tuning(solo_max_edges=edges, grid_blocks=blocks)
+                dist, st, settle, _ = sp.solve_trace(G, 1, sp.IN_OUT)
+                assert (sp.as_uint64(dist) == ref).all() and (settle == sim.settle_phase).all(), (g.name, blocks)
+                assert (st["settled"], st["edges_relaxed"]) == (sim.settled, sim.relaxed)
+                dist, phases = sp.solve(G, 1, sp.IN_OUT)
+                assert (sp.as_uint64(dist) == ref).all() and phases == sim.phases, (g.name, blocks)
+    finally:
+        sp.set_tuning()
