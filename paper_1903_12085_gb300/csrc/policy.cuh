@@ -43,29 +43,32 @@ constexpr int kPolOffW3 = kPolOffB2 + kPolHidden;
 constexpr int kPolOffB3 = kPolOffW3 + kPolHidden * kPolArms;
 constexpr int kPolWeights = kPolOffB3 + kPolArms;  // 1476
 
-__host__ __device__ __forceinline__ void policy_features(float* f, uint64_t nF, uint64_t n, uint64_t m, uint64_t k,
-                                                         uint64_t e_prev, uint64_t s_prev, uint64_t f_prev) {
-  f[0] = log2f(1.0f + (float)nF) / 24.0f;
-  f[1] = (float)nF / (float)n;
-  f[2] = log2f(1.0f + (float)e_prev) / 24.0f;
-  f[3] = log2f(1.0f + (float)s_prev) / 24.0f;
-  f[4] = log2f(1.0f + (float)k) / 16.0f;
-  f[5] = log2f((float)n) / 32.0f;
-  f[6] = ((float)m / (float)n) / 32.0f;
-  f[7] = (float)s_prev / (1.0f + (float)f_prev);
+// Feature i from the counts above, as float32: the one formula, for the host
+// (policy_features) and for the engine's warps (policy_feature_lane), which have
+// one logarithm and one division in a row this way instead of five and eight.
+// (A scale by a power of two is exact, before or after.)
+__host__ __device__ __forceinline__ float policy_feature(int i, float nF, float n, float m, float k, float e_prev,
+                                                         float s_prev, float f_prev) {
+  const float x = i == 0 || i == 1 ? nF : i == 2 ? e_prev : i == 4 ? k : i == 5 ? n : i == 6 ? m : s_prev;
+  const float num = i < 6 && i != 1 ? log2f(i == 5 ? x : 1.0f + x) : x;
+  const float den = i == 1 || i == 6 ? n : i == 7 ? 1.0f + f_prev : i == 4 || i == 5 ? 1.0f : 24.0f;
+  const float scale = i == 4 ? 1.0f / 16.0f : i == 5 || i == 6 ? 1.0f / 32.0f : 1.0f;
+  return num / den * scale;
 }
 
-// The same features by one full warp, feature i in lane i (i < 8; other lanes: 0):
-// one logarithm and one division in a row instead of five and eight, with the
-// same results (a scale by a power of two is exact, before or after).
+__host__ __device__ __forceinline__ void policy_features(float* f, uint64_t nF, uint64_t n, uint64_t m, uint64_t k,
+                                                         uint64_t e_prev, uint64_t s_prev, uint64_t f_prev) {
+  for (int i = 0; i < kPolFeat; ++i)
+    f[i] = policy_feature(i, (float)nF, (float)n, (float)m, (float)k, (float)e_prev, (float)s_prev, (float)f_prev);
+}
+
+// The same by one full warp, feature i in lane i (i < 8; other lanes: 0).
 __device__ __forceinline__ float policy_feature_lane(uint32_t nF, uint32_t n, uint32_t m, uint32_t k,
                                                      uint32_t e_prev, uint32_t s_prev, uint32_t f_prev) {
   const int i = threadIdx.x & 31;
-  const float x = (float)(i == 0 || i == 1 ? nF : i == 2 ? e_prev : i == 4 ? k : i == 5 ? n : i == 6 ? m : s_prev);
-  const float num = i < 6 && i != 1 ? log2f(i == 5 ? x : 1.0f + x) : x;
-  const float den = i == 1 || i == 6 ? (float)n : i == 7 ? 1.0f + (float)f_prev : i == 4 || i == 5 ? 1.0f : 24.0f;
-  const float scale = i == 4 ? 1.0f / 16.0f : i == 5 || i == 6 ? 1.0f / 32.0f : 1.0f;
-  return i < kPolFeat ? num / den * scale : 0.0f;
+  const float f =
+      policy_feature(i, (float)nF, (float)n, (float)m, (float)k, (float)e_prev, (float)s_prev, (float)f_prev);
+  return i < kPolFeat ? f : 0.0f;
 }
 
 // Place of weight i in a block's shared-memory copy: the matrices of the hidden
