@@ -53,6 +53,7 @@ struct GraphView {
   const uint2* redges;       // [m] {source, cost}, rows sorted by (cost, source)
   const uint2* rowdeg;       // [n] {start of out-row, out-degree} (m < 2^32)
   uint32_t max_w;            // largest edge cost (0 without edges)
+  uint32_t max_deg;          // largest out-degree
 };
 
 // Per-vertex record gathered by the selection and relax steps: the tentative

@@ -2745,16 +2745,24 @@ __global__ void __launch_bounds__(kT, kThreads / kT) k_solve_batch(const BatchIt
 // ---------------------------------------------------------------------------
 // host side
 
-// Graphs of at most kSoloLargeN vertices, or with fewer than 6 edges a vertex
-// (meshes and the like, whose fringes stay small for many phases), get twice the
-// slots: their solves live in episodes.  On larger and denser ones the grid
-// phases count, and these want the L1 that the slots would take.  (G(2^14, 2^17)
-// with 4, 8, 12, 16 slots a thread: 1.47, 1.37, 1.43, 1.64 ms; the 1024 x 1024
-// grid 110.7, 108.9, 110.4, 110.3.)  In blocks of kSmallThreads, two to an SM,
-// the meshes alone: 200 solves of G(20000, 160000) take 5.5 ms with 16 slots a
-// thread, 4.2 with 8, and 256 sources on the 512 x 512 grid 48 and 73.
-static bool solo_mesh(uint32_t n, uint64_t m) { return m < 6ull * n; }
-static bool solo_large(uint32_t n, uint64_t m) { return n <= kSoloLargeN || solo_mesh(n, m); }
+// Graphs of at most kSoloLargeN vertices, and meshes, get twice the slots: their
+// solves live in episodes.  On other graphs the grid phases count, and these want
+// the L1 that the slots would take (G(2^22, 4.7 x 2^22) 18.2 ms with 8 slots a
+// thread and 17.7 with 4, R-MAT of 2^20 vertices 3.57 and 3.51; the 1024 x 1024
+// grid with 4, 8, 12, 16 slots 271, 109, 111, 112 ms, since 4 cannot hold its
+// fringe; G(2^14, 2^17) 1.18, 1.11, 1.15, 1.38).  In blocks of kSmallThreads, two to an SM, the meshes alone: 250 solves of G(100000, 470000)
+// take 25.4 ms with 16 slots a thread, 16.4 with 8, of G(3000, 16500) 0.80 and
+// 0.85, and 256 sources on the 512 x 512 grid 44 and 73.
+//
+// A mesh: a graph without a row of more than kMeshDegree edges, whose searches
+// grow by a few vertices at a time.  Grids with 4 and with 8 neighbours are, and
+// road networks; uniform and R-MAT graphs have longer rows at any density from 2
+// edges a vertex on.  (By the density alone, below 6 edges a vertex, sparse
+// uniform and R-MAT graphs counted as meshes and the grid with 8 neighbours did
+// not: 1024 x 1024 of those 366 ms, now 211.)
+constexpr uint32_t kMeshDegree = 8;
+static bool solo_mesh(const GraphView& g) { return g.max_deg <= kMeshDegree; }
+static bool solo_large(const GraphView& g) { return g.n <= kSoloLargeN || solo_mesh(g); }
 
 // The kernel instance for a criterion mask (see kAny).
 int kind_of(uint32_t crit, bool narrow, bool records) {
@@ -2881,7 +2889,7 @@ size_t solo_shape_of(bool large, bool narrow, uint32_t crit, uint32_t threads, P
 }  // namespace
 
 size_t solo_shape(uint32_t crit, SolveParams* p) {
-  return solo_shape_of(solo_large(p->g.n, p->g.m), p->g.max_w <= kSoloNarrowW, crit, kThreads, p);
+  return solo_shape_of(solo_large(p->g), p->g.max_w <= kSoloNarrowW, crit, kThreads, p);
 }
 
 void workspace_free(Workspace* ws) {
@@ -3050,13 +3058,17 @@ sssp_status solve_one(sssp_graph* g, uint32_t source, uint32_t crit, uint64_t* d
 struct BatchPlan {
   uint32_t count = 0;
   uint32_t crit = 0;
-  bool large = true, mesh = true, narrow = true;  // see solo_shape_of
+  // see solo_shape_of; deep: a mesh whose fringe needs the slots is among the
+  // graphs, which then all get them (they cost the others 1 to 3 %)
+  bool large = true, mesh = true, narrow = true, deep = false;
+  bool light = true;                   // see kind
   uint32_t recording = 0;              // solves with a trace or settle phases attached
-  // Policy solves of graphs with small episodes (solo_large) run mostly grid
-  // phases, whose steps spill least in the batch's general instance: 8 sources of
-  // G(2^24, 2^28) at once 117 ms, in the policy's own 122.  (Single solves are
-  // the other way round: G(2^20, 2^24) 8.6 and 8.0 ms.)
-  int kind() const { return kind_of(crit, narrow, recording != 0 || (!large && (crit & SSSP_POLICY_LEARNED))); }
+  // Policy solves of large and dense graphs run mostly grid phases, whose steps
+  // spill least in the batch's general instance: 8 sources of G(2^24, 2^28) at
+  // once 117 ms, in the policy's own 122; 12 of a sparse R-MAT graph (`light`:
+  // fewer than 6 edges a vertex) of 2^20 vertices 6.27 and 6.10.  (Single solves
+  // are the other way round: G(2^20, 2^24) 8.6 and 8.0 ms.)
+  int kind() const { return kind_of(crit, narrow, recording != 0 || (!light && (crit & SSSP_POLICY_LEARNED))); }
   BatchTuning tuning{};                // in force when the batch was created (or autotuned last)
   unsigned long long wait_ns = 0;      // the wait limit then
   uint32_t bpg = 1;                    // blocks per solve
@@ -3106,8 +3118,9 @@ void batch_free(sssp_batch* b) {
 // to 2^18 vertices) with one source each 37.6 -> 24.6 ms, with four each, where
 // only the largest few are above the share, 53 -> 51.7 ms.  With a half or a
 // quarter of the share as the limit, four sources take 54 and 60 ms.  Meshes
-// keep to one block, which runs their small fringes fastest, and a policy's
-// batches to one size, on which its choices depend.
+// keep to one block, to which more add nothing (four 724 x 724 grids 66.1, 65.4,
+// 66.9 and 66.6 ms with 1, 2, 4 and 16 blocks each), and a policy's batches to
+// one size, on which its choices depend.
 //
 // More solves than SMs and of about one size (the largest at most twice the
 // mean) run in blocks of kSmallThreads, two to an SM, whose latency chains
@@ -3171,7 +3184,7 @@ sssp_status batch_enqueue(sssp_batch* b, cudaStream_t st) {
   SSSP_CUDA_TRY(cudaMemsetAsync(b->err, 0, sizeof(int), st));
   for (Workspace* w : b->ws) SSSP_CUDA_TRY(cudaMemsetAsync(w->ctl, 0, sizeof(Ctl), st));
   BatchTuning tu = b->tuning;
-  const size_t smem = solo_shape_of(l.threads == kThreads ? b->large : b->mesh, b->narrow, b->crit, l.threads, &tu);
+  const size_t smem = solo_shape_of(l.threads == kThreads ? b->large || b->deep : b->mesh, b->narrow, b->crit, l.threads, &tu);
   void* args[] = {&b->items, &b->next, &b->gslots, &l.stages, &b->crit, &tu, &b->wait_ns, &b->err, &b->phases, &b->policy};
   SSSP_CUDA_TRY(cudaLaunchCooperativeKernel(batch_kernel(b->kind(), l.threads), dim3(l.blocks), dim3(l.threads), args,
                                             smem, st));
@@ -3210,9 +3223,12 @@ sssp_status batch_build(sssp_graph* const* graphs, const uint32_t* sources, uint
   b->count = count;
   b->crit = crit;
   for (uint32_t i = 0; i < count; ++i) {
-    b->large = b->large && solo_large(graphs[i]->n, graphs[i]->m);
-    b->mesh = b->mesh && solo_mesh(graphs[i]->n, graphs[i]->m);
-    b->narrow = b->narrow && graphs[i]->max_w <= kSoloNarrowW;
+    const GraphView g = view_of(graphs[i]);
+    b->large = b->large && solo_large(g);
+    b->mesh = b->mesh && solo_mesh(g);
+    b->deep = b->deep || (solo_mesh(g) && g.n > kSoloLargeN);
+    b->light = b->light && (g.n <= kSoloLargeN || g.m < 6ull * g.n);
+    b->narrow = b->narrow && g.max_w <= kSoloNarrowW;
   }
   b->bpg = bpg;
   b->staged = !tuned && bpg == 1;

@@ -264,15 +264,18 @@ __global__ void k_fill_u32(uint32_t* p, uint64_t n, uint32_t v) {
 
 __global__ void k_out_min(const uint64_t* __restrict__ ro, const uint2* __restrict__ edges, uint32_t n,
                           uint32_t* __restrict__ out_min, uint2* __restrict__ rowdeg,
-                          unsigned int* __restrict__ max_w) {
-  uint32_t top = 0;  // (the last edge of a sorted row is its dearest)
+                          unsigned int* __restrict__ tops) {
+  uint32_t top = 0, deg = 0;  // (the last edge of a sorted row is its dearest)
   for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
     out_min[u] = ro[u + 1] > ro[u] ? edges[ro[u]].y : kInf32;
     rowdeg[u] = make_uint2((uint32_t)ro[u], (uint32_t)(ro[u + 1] - ro[u]));
     if (ro[u + 1] > ro[u]) top = max(top, edges[ro[u + 1] - 1].y);
+    deg = max(deg, (uint32_t)(ro[u + 1] - ro[u]));
   }
   top = __reduce_max_sync(0xFFFFFFFFu, top);
-  if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(max_w, top);
+  deg = __reduce_max_sync(0xFFFFFFFFu, deg);
+  if ((threadIdx.x & 31) == 0 && top > 0) atomicMax(&tops[0], top);
+  if ((threadIdx.x & 31) == 0 && deg > 0) atomicMax(&tops[1], deg);
 }
 
 __global__ void k_in_min(const uint2* __restrict__ edges, uint64_t m, uint32_t* __restrict__ in_min) {
@@ -503,11 +506,11 @@ sssp_status build(sssp_graph* g, const uint64_t* ro_in, const uint32_t* col_in, 
   }
   s = sort_rows(g->row_off, n, m, reinterpret_cast<unsigned long long*>(g->edges), st);
   if (s != SSSP_OK) return s;
-  TmpBuf<unsigned int> wbuf(st);
-  if ((s = wbuf.alloc(1)) != SSSP_OK) return s;
-  SSSP_CUDA_TRY(cudaMemsetAsync(wbuf.p, 0, sizeof(unsigned int), st));
-  k_out_min<<<grid_for(n, 256), 256, 0, st>>>(g->row_off, g->edges, n, g->out_min, g->rowdeg, wbuf.p);
-  SSSP_CUDA_TRY(cudaMemcpyAsync(&g->max_w, wbuf.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  TmpBuf<unsigned int> tops(st);  // {largest cost, largest out-degree}
+  if ((s = tops.alloc(2)) != SSSP_OK) return s;
+  SSSP_CUDA_TRY(cudaMemsetAsync(tops.p, 0, 2 * sizeof(unsigned int), st));
+  k_out_min<<<grid_for(n, 256), 256, 0, st>>>(g->row_off, g->edges, n, g->out_min, g->rowdeg, tops.p);
+  SSSP_CUDA_TRY(cudaMemcpyAsync(g->tops, tops.p, sizeof(g->tops), cudaMemcpyDeviceToHost, st));
   k_fill_u32<<<grid_for(n, 256), 256, 0, st>>>(g->in_min, n, kInf32);
   if (m > 0) k_in_min<<<grid_for(m, 256), 256, 0, st>>>(g->edges, m, g->in_min);
   SSSP_CUDA_TRY(cudaGetLastError());
@@ -544,7 +547,8 @@ GraphView view_of(const sssp_graph* g) {
   v.out_min = g->out_min;
   v.in_min = g->in_min;
   v.rowdeg = g->rowdeg;
-  v.max_w = g->max_w;
+  v.max_w = g->tops[0];
+  v.max_deg = g->tops[1];
   v.rrow_off = g->rrow_off;
   v.redges = g->redges;
   return v;

@@ -98,7 +98,7 @@ struct sssp_graph {
   uint32_t* out_min;   // device [n]
   uint32_t* in_min;    // device [n]
   uint2* rowdeg;       // device [n] {row start, out-degree}
-  uint32_t max_w;      // largest edge cost
+  uint32_t tops[2];    // largest edge cost, largest out-degree
   uint64_t* rrow_off;  // device [n+1] or nullptr
   uint2* redges;       // device [m] or nullptr
   // Lazily allocated solve workspace (shared by solves on this handle).

@@ -82,8 +82,8 @@ __global__ void k_noalloc_minima_init(uint32_t n, uint32_t* out_min, uint32_t* i
 // (bad[0] set on an out-of-range target, a reserved cost or bad offsets).
 __global__ void k_noalloc_minima(uint32_t n, uint64_t m, const uint64_t* __restrict__ ro,
                                  const uint2* __restrict__ edges, uint32_t* out_min, uint32_t* in_min,
-                                 uint2* rowdeg, int* bad, unsigned int* max_w) {
-  uint32_t top = 0;
+                                 uint2* rowdeg, int* bad, unsigned int* max_w, unsigned int* max_deg) {
+  uint32_t top = 0, deg = 0;
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t warp0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -108,10 +108,12 @@ __global__ void k_noalloc_minima(uint32_t n, uint64_t m, const uint64_t* __restr
     if (lane == 0) {
       out_min[u] = best;
       rowdeg[u] = make_uint2((uint32_t)b, (uint32_t)(e - b));
+      deg = max(deg, (uint32_t)(e - b));
     }
   }
   top = __reduce_max_sync(0xFFFFFFFFu, top);
   if (lane == 0 && top > 0) atomicMax(max_w, top);
+  if (lane == 0 && deg > 0) atomicMax(max_deg, deg);
 }
 
 }  // namespace
@@ -157,12 +159,13 @@ extern "C" sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t
   const int blocks = dev->max_blocks;
   k_noalloc_minima_init<<<blocks, 256, 0, st>>>(n, out_min, in_min);
   k_noalloc_minima<<<blocks, 256, 0, st>>>(n, m, row_offsets, e2, out_min, in_min, rowdeg, &ctl->err,
-                                          &ctl->nf_tmp);  // (a free word of the block)
+                                          &ctl->nf_tmp, &ctl->nf_moved);  // (free words of the block)
   SSSP_CUDA_TRY(cudaGetLastError());
   int bad = 0;
-  uint32_t max_w = 0;
+  uint32_t max_w = 0, max_deg = 0;
   SSSP_CUDA_TRY(cudaMemcpyAsync(&bad, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   SSSP_CUDA_TRY(cudaMemcpyAsync(&max_w, &ctl->nf_tmp, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  SSSP_CUDA_TRY(cudaMemcpyAsync(&max_deg, &ctl->nf_moved, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   SSSP_CUDA_TRY(cudaStreamSynchronize(st));
   if (bad) return fail(SSSP_ERR_INVALID_ARG, "sssp_solve_noalloc: invalid CSR (offsets, targets or costs)");
   SSSP_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
@@ -177,6 +180,7 @@ extern "C" sssp_status sssp_solve_noalloc(uint32_t n, uint64_t m, const uint64_t
   p.g.in_min = in_min;
   p.g.rowdeg = rowdeg;
   p.g.max_w = max_w;
+  p.g.max_deg = max_deg;
   p.ws.dist = reinterpret_cast<unsigned long long*>(dist_out);
   p.ws.vrec = reinterpret_cast<VRec*>(base + kOffVrec);
   p.ws.status = base + kOffStatus;
