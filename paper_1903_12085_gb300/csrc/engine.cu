@@ -2750,14 +2750,15 @@ __global__ void __launch_bounds__(kT, kThreads / kT) k_solve_batch(const BatchIt
 // the L1 that the slots would take (G(2^22, 4.7 x 2^22) 18.2 ms with 8 slots a
 // thread and 17.7 with 4, R-MAT of 2^20 vertices 3.57 and 3.51; the 1024 x 1024
 // grid with 4, 8, 12, 16 slots 271, 109, 111, 112 ms, since 4 cannot hold its
-// fringe; G(2^14, 2^17) 1.18, 1.11, 1.15, 1.38).  In blocks of kSmallThreads, two to an SM, the meshes alone: 250 solves of G(100000, 470000)
-// take 25.4 ms with 16 slots a thread, 16.4 with 8, of G(3000, 16500) 0.80 and
-// 0.85, and 256 sources on the 512 x 512 grid 44 and 73.
+// fringe; G(2^14, 2^17) 1.18, 1.11, 1.15, 1.38).  In blocks of kSmallThreads, two
+// to an SM, the meshes alone: 250 solves of G(100000, 470000) take 25.4 ms with 16
+// slots a thread, 16.4 with 8, of G(3000, 16500) 0.80 and 0.85, and 256 sources
+// on the 512 x 512 grid 44 and 73.
 //
 // A mesh: a graph without a row of more than kMeshDegree edges, whose searches
 // grow by a few vertices at a time.  Grids with 4 and with 8 neighbours are, and
-// road networks; uniform and R-MAT graphs have longer rows at any density from 2
-// edges a vertex on.  (By the density alone, below 6 edges a vertex, sparse
+// road networks; uniform and R-MAT graphs have longer rows from 4 edges a vertex
+// on, the thousand vertices of the smallest included.  (By the density alone, below 6 edges a vertex, sparse
 // uniform and R-MAT graphs counted as meshes and the grid with 8 neighbours did
 // not: 1024 x 1024 of those 366 ms, now 211.)
 constexpr uint32_t kMeshDegree = 8;
